@@ -347,9 +347,11 @@ void choose_tiles(gg_plan_t *plan) {
   int cap = gg::max_block_threads_axis<R>(e);
   if (cap <= 0) cap = 256;
   while (b > 1 && (n / e) * b > std::min(cap, 512)) b /= 2;
-  int rows = 1;
+  // box height: every box of a tile must start on a 128-byte boundary of shared
+  // memory (N = 324 with 16-byte rows has no such divisor: plain loads there)
+  int rows = 0;
   for (int d = 1; d <= 256 && d <= n; ++d)
-    if (n % d == 0) rows = d;
+    if (n % d == 0 && (d == n || (size_t)d * b * cb % 128 == 0)) rows = d;
   plan->col_b = b;
   plan->col_e = e;
   plan->col_rows_box = (sizeof(R) == 8 || half % 2 == 0) && (size_t)b * cb >= 16 ? rows : 0;

@@ -1,0 +1,40 @@
+"""Grid sizes off the tuned list against the oracle: sizes whose strided tiles
+take several TMA boxes of narrow rows (each box must start on a 128-byte
+boundary of shared memory).
+
+Tolerances as in test_gpu_parity: 1e-5 (FP32) and 1e-12 (FP64) relative L2.
+"""
+import pytest
+
+from tests.gpu_helpers import rel_l2, run_oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+BBKS = dict(omega_m=0.3, h=0.7, n_s=0.96, sigma_8=0.8, tf="bbks", omega_l=-1.0,
+            omega_b=0.049, t_cmb=2.7255)
+
+
+@pytest.fixture(scope="module")
+def gg():
+    from paper_2511_10353_gb300 import build
+    build.build(verbose=False)
+    import paper_2511_10353_gb300 as m
+    return m
+
+
+def check(gg, n, prec):
+    plan = gg.Plan(n, float(n), BBKS, 50.0, prec)
+    out = plan.zeldovich(seed=5, pos=False)
+    plan.sync()
+    ora = run_oracle(dict(n=n, box=float(n), cosmo=BBKS, z_init=50.0), seed=5)
+    tol = 1e-12 if prec == "f64" else 1e-5
+    for k in ("psi", "vel"):
+        for j in range(3):
+            assert rel_l2(out[k][j].cpu().numpy(), ora[k][j]) < tol, (k, j)
+    plan.close()
+
+
+@pytest.mark.parametrize("prec", ["f32", "f64"])
+def test_narrow_rows_in_several_boxes(gg, prec):
+    check(gg, 324, prec)
