@@ -194,7 +194,8 @@ gg_status gg_profile_read(gg_plan_t *plan, int reset, int *count, const char **n
                           int64_t *launches, double *bytes);
 
 /* Autotuner of the transform tiles (grid sizes with size-specialised kernels:
- * N = 64, 128, 192, 256, 384, 512, 1536 in FP32; 64, 512, 1536 in FP64).
+ * N = 64, 128, 192, 256, 384, 512, 1536 in FP32; 64, 512, 1536 in FP64; the
+ * other specialised sizes have one tile shape).
  * Runs the whole path `reps` times per tile variant on the plan's own buffers
  * (allocating the component workspaces and one scratch grid for the call),
  * times each pass with CUDA events and keeps the fastest variant per pass for

@@ -860,7 +860,7 @@ gg_status run_host(gg_plan_t *plan, uint64_t seed, const void *noise_host, void 
 // kind map below picks each pass's time.
 template <typename R>
 gg_status autotune(gg_plan_t *plan, int reps) {
-  if (!gg::spec_has<R>((int)plan->p.n)) return GG_OK;
+  if (!gg::spec_tuned<R>((int)plan->p.n)) return GG_OK;
   gg_status st;
   if ((st = ensure_grid(plan, &plan->work2)) != GG_OK) return st;
   if ((st = ensure_grid(plan, &plan->work3)) != GG_OK) return st;

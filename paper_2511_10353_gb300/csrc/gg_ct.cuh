@@ -39,9 +39,28 @@ __host__ __device__ constexpr Fac factor(int n) {
   while (n % 3 == 0) { n /= 3; ++f.b; }
   return f;
 }
-// large-radix forward schedules of the FP32 codelets (0: none at this n / stage)
+// large-radix forward schedules of the FP32 codelets (0: none at this n / stage).
+// Two stages of radices up to 24 where the length splits that way, else three
+// of radices up to 16 (one at 18): few shared-memory round trips, at most 24
+// elements a thread (32 at 512). 1024 = 16 x 16 x 4 keeps 16 elements a
+// thread, so that a 512-thread CTA holds the spectrum in registers.
 __host__ __device__ constexpr int big_radix(int n, int s) {
   switch (n) {
+    case 24: return s == 0 ? 4 : (s == 1 ? 6 : 0);
+    case 36: return s < 2 ? 6 : 0;
+    case 48: return s == 0 ? 4 : (s == 1 ? 12 : 0);
+    case 72: return s == 0 ? 6 : (s == 1 ? 12 : 0);
+    case 108: return s < 2 ? 6 : (s == 2 ? 3 : 0);
+    case 144: return s < 2 ? 12 : 0;
+    case 216: return s < 3 ? 6 : 0;
+    case 288: return s == 0 ? 12 : (s == 1 ? 24 : 0);
+    case 324: return s < 2 ? 6 : (s == 2 ? 9 : 0);
+    case 432: return s < 2 ? 6 : (s == 2 ? 12 : 0);
+    case 576: return s < 2 ? 24 : 0;
+    case 648: return s < 2 ? 6 : (s == 2 ? 18 : 0);
+    case 864: return s == 0 ? 6 : (s < 3 ? 12 : 0);
+    case 1024: return s < 2 ? 16 : (s == 2 ? 4 : 0);
+    case 1152: return s == 0 ? 8 : (s < 3 ? 12 : 0);
     case 256: return s < 2 ? 16 : 0;
     case 512: return s == 0 ? 32 : (s == 1 ? 16 : 0);
     case 768: return s < 2 ? 8 : (s == 2 ? 12 : 0);
@@ -202,8 +221,10 @@ template <int R1, int R2, bool INV, typename T> struct ComposedDft {
   }
 };
 template <bool INV, typename T> struct Butterfly<6, INV, T> : ComposedDft<2, 3, INV, T> {};
+template <bool INV, typename T> struct Butterfly<9, INV, T> : ComposedDft<3, 3, INV, T> {};
 template <bool INV, typename T> struct Butterfly<12, INV, T> : ComposedDft<4, 3, INV, T> {};
 template <bool INV, typename T> struct Butterfly<16, INV, T> : ComposedDft<4, 4, INV, T> {};
+template <bool INV, typename T> struct Butterfly<18, INV, T> : ComposedDft<6, 3, INV, T> {};
 template <bool INV, typename T> struct Butterfly<24, INV, T> : ComposedDft<8, 3, INV, T> {};
 template <bool INV, typename T> struct Butterfly<32, INV, T> : ComposedDft<8, 4, INV, T> {};
 template <bool INV, typename T> struct Butterfly<48, INV, T> : ComposedDft<16, 3, INV, T> {};
@@ -509,7 +530,15 @@ __device__ __forceinline__ void inverse_head_store(int p, const Cx<R> *v, const 
 // threads per CTA for every pass and size, two CTAs per SM.
 constexpr int kPersistV = 4;
 
+// Sizes with several tile variants for the autotuner (the named workloads'
+// and their neighbours); every other size has the one shape of variant 0.
+template <typename R> __host__ __device__ constexpr bool ct_tuned(int n) {
+  if (sizeof(R) == 8) return n == 64 || n == 512 || n == 1536;
+  return n == 64 || n == 128 || n == 192 || n == 256 || n == 384 || n == 512 || n == 1536;
+}
+
 template <typename R, int N, int V> struct AxisPolicy {
+  static constexpr bool TUNED = ct_tuned<R>(N);
   static constexpr int CB = 2 * (int)sizeof(R);
   static constexpr bool BIG = is_big(skey<R>(N));
   static constexpr int E0 = elems(skey<R>(N));
@@ -523,7 +552,7 @@ template <typename R, int N, int V> struct AxisPolicy {
   static constexpr int pick() {
     if (V == kPersistV) return 256 / P;  // the persistent batched kernel: 256 threads
     int b = 128 / CB;
-    while (b > 1 && ((N / 2) % b != 0 || P * b > 512 || 2 * (N * b * CB) > 200 * 1024)) b /= 2;
+    while (b > 1 && ((N / 2) % b != 0 || P * b > (TUNED ? 512 : 640) || 2 * (N * b * CB) > 200 * 1024)) b /= 2;
     if (SMALL && b * CB > 32) b /= 2;
     return b;
   }
@@ -543,9 +572,16 @@ template <typename R, int N, int V> struct AxisPolicy {
   static constexpr bool THREE = V == 2 && BIG && sizeof(R) == 4 && N >= 512 &&
                                 3 * (SMEM_EST + 4 * kInterpExact + 16 * kMaxInterpCells(N) + 1024) <=
                                     228 * 1024;
+  static constexpr int REG_NEED = 4 * E * ((int)sizeof(R) / 4) + 48;
   static constexpr int min_blocks() {
     if (V == kPersistV) return 2;
     if (THREE) return 3;
+    if (!TUNED) {  // as many CTAs as shared memory and the register estimate allow
+      const int by_smem = (228 * 1024) / (SMEM_EST + N * CB + 4 * kInterpExact + 16 * kMaxInterpCells(N) + 1024);
+      const int by_regs = 65536 / (THREADS * (REG_NEED + 8));
+      const int m = by_smem < by_regs ? by_smem : by_regs;
+      return m < 1 ? 1 : (m > 8 ? 8 : m);
+    }
     if (BIG && V == 1) {  // the x pass's filter table (about 11 KB) may still cost one
       const int by_smem = (228 * 1024) / (SMEM_EST + 1024);
       return by_smem < 1 ? 1 : (by_smem > 3 ? 3 : by_smem);
@@ -555,9 +591,17 @@ template <typename R, int N, int V> struct AxisPolicy {
   static constexpr int MINB = min_blocks();
   static constexpr int REG_BUDGET =
       65536 / (THREADS * MINB) < 255 ? 65536 / (THREADS * MINB) : 255;
-  static constexpr int REG_NEED = 4 * E * ((int)sizeof(R) / 4) + 48;
   static constexpr bool SPILL = (BIG && V == 1) || (!THREE && REG_NEED > REG_BUDGET);
-  static constexpr int ROWS_BOX = N <= 256 ? N : (N % 256 == 0 ? 256 : (N % 192 == 0 ? 192 : 128));
+  // TMA box height: the largest divisor of N up to 256 whose boxes start on
+  // 128-byte boundaries of shared memory
+  static constexpr int rows_box() {
+    int rows = 0;
+    for (int d = 1; d <= 256 && d <= N; ++d)
+      if (N % d == 0 && (d == N || d * B * CB % 128 == 0)) rows = d;
+    return rows;
+  }
+  static constexpr int ROWS_BOX = rows_box();
+  static_assert(ROWS_BOX > 0, "no TMA box height");
   static_assert(V != kPersistV || (THREADS == 256 && (N / 2) % B == 0), "persistent tile");
   // the large radices read their stage twiddles from a shared-memory copy
   // where it fits beside the tiles and the largest filter table

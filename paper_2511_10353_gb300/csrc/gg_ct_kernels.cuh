@@ -50,7 +50,7 @@ __host__ __device__ constexpr bool axis_tma_store_fwd() {
 template <typename R, int N, int V, int MODE, bool CUT = false, int FILT = kFiltArgs>
 __host__ __device__ constexpr bool axis_tma_store_inplace() {
   using Pol = ct::AxisPolicy<R, N, V>;
-  return MODE != kAxisFwd && (Pol::SPILL || Pol::THREE) && V != ct::kPersistV &&
+  return MODE != kAxisFwd && (Pol::SPILL || Pol::THREE || !Pol::TUNED) && V != ct::kPersistV &&
          ct::nstages(ct::skey<R>(N)) > 1 &&
          !ct::fuse_pair<R, N, Pol::E>() && !axis_tma_store<R, N, V, MODE, CUT, FILT>();
 }
@@ -813,7 +813,8 @@ constexpr int kZVariants = 4;
 template <typename R, int... NS> struct CtTable {
   static bool has(int n) { return ((n == NS) || ...); }
   template <int N> static int cols_n(int v) {
-    return v == 1 ? ct::AxisPolicy<R, N, 1>::B : (v == 2 ? ct::AxisPolicy<R, N, 2>::B : ct::AxisPolicy<R, N, 0>::B);
+    if constexpr (!ct::ct_tuned<R>(N)) return ct::AxisPolicy<R, N, 0>::B;
+    else return v == 1 ? ct::AxisPolicy<R, N, 1>::B : (v == 2 ? ct::AxisPolicy<R, N, 2>::B : ct::AxisPolicy<R, N, 0>::B);
   }
   static int cols(int n, int v) {
     int c = 0;
@@ -840,7 +841,11 @@ template <typename R, int... NS> struct CtTable {
       if (!(a.fwd && a.inv)) return cudaErrorInvalidValue;
       return ct_launch_axis<R, N, 0, kAxisFwdInv, true>(a, s);
     }
-    return a.variant == 1 ? axis_v<N, 1>(a, s) : (a.variant == 2 ? axis_v<N, 2>(a, s) : axis_v<N, 0>(a, s));
+    if constexpr (ct::ct_tuned<R>(N)) {
+      if (a.variant == 1) return axis_v<N, 1>(a, s);
+      if (a.variant == 2) return axis_v<N, 2>(a, s);
+    }
+    return axis_v<N, 0>(a, s);
   }
   static cudaError_t axis(const AxisArgs &a, cudaStream_t s) {
     cudaError_t e = cudaErrorInvalidValue;
@@ -865,20 +870,20 @@ template <typename R, int... NS> struct CtTable {
   template <int N> static cudaError_t zinv_n(const ZInvArgs &a, cudaStream_t s) {
     if (a.large || a.pos2 || a.shift != 0.0 || a.shift2 != 0.0)  // Secs. 2.2, 2.4 options: variant 0
       return ct_launch_zinv<R, N, 0, true>(a, s);
-    switch (a.variant) {
-      case 1: return zinv_v<N, 1>(a, s);
-      case 2: return zinv_v<N, 2>(a, s);
-      case 3: return zinv_v<N, 3>(a, s);
-      default: return zinv_v<N, 0>(a, s);
+    if constexpr (ct::ct_tuned<R>(N)) {
+      if (a.variant == 1) return zinv_v<N, 1>(a, s);
+      if (a.variant == 2) return zinv_v<N, 2>(a, s);
+      if (a.variant == 3) return zinv_v<N, 3>(a, s);
     }
+    return zinv_v<N, 0>(a, s);
   }
   template <int N> static cudaError_t zfwd_n(const ZFwdArgs &a, cudaStream_t s) {
-    switch (a.variant) {
-      case 1: return ct_launch_zfwd<R, N, 1>(a, s);
-      case 2: return ct_launch_zfwd<R, N, 2>(a, s);
-      case 3: return ct_launch_zfwd<R, N, 3>(a, s);
-      default: return ct_launch_zfwd<R, N, 0>(a, s);
+    if constexpr (ct::ct_tuned<R>(N)) {
+      if (a.variant == 1) return ct_launch_zfwd<R, N, 1>(a, s);
+      if (a.variant == 2) return ct_launch_zfwd<R, N, 2>(a, s);
+      if (a.variant == 3) return ct_launch_zfwd<R, N, 3>(a, s);
     }
+    return ct_launch_zfwd<R, N, 0>(a, s);
   }
   static cudaError_t zinv(const ZInvArgs &a, cudaStream_t s) {
     cudaError_t e = cudaErrorInvalidValue;

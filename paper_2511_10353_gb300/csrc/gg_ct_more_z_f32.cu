@@ -1,0 +1,10 @@
+// F32 size-specialised kernels, z passes, of the sizes in gg_ct_more_f32.cu.
+#include "gg_ct_kernels.cuh"
+
+namespace gg {
+
+using MoreF32 = CtTable<float, GG_MORE_F32>;
+cudaError_t spec_more_zinv_f32(const ZInvArgs &a, cudaStream_t s) { return MoreF32::zinv(a, s); }
+cudaError_t spec_more_zfwd_f32(const ZFwdArgs &a, cudaStream_t s) { return MoreF32::zfwd(a, s); }
+
+}  // namespace gg

@@ -234,6 +234,14 @@ template <typename R> int max_block_threads_axis(int e);
 // Size-specialised kernels (gg_ct_f32.cu / gg_ct_f64.cu) for the grid sizes of
 // the named workloads; spec_has tells whether N has them.
 template <typename R> bool spec_has(int n);
+template <typename R> bool spec_tuned(int n);  // has tile variants (gg_autotune)
+// the F32 sizes with one tile shape (gg_ct_more_f32.cu, gg_ct_more_z_f32.cu)
+#define GG_MORE_F32 32, 48, 72, 96, 144, 216, 288, 432, 576, 648, 768, 864, 1024, 1152
+bool spec_more_has_f32(int n);
+int spec_more_cols_f32(int n, int v);
+cudaError_t spec_more_axis_f32(const AxisArgs &a, cudaStream_t s);
+cudaError_t spec_more_zinv_f32(const ZInvArgs &a, cudaStream_t s);
+cudaError_t spec_more_zfwd_f32(const ZFwdArgs &a, cudaStream_t s);
 constexpr int kSpecAxisVariants = 3;  // tile variants the autotuner times per strided pass
 constexpr int kSpecZVariants = 4;     // ... per z pass
 template <typename R> cudaError_t spec_axis(const AxisArgs &a, cudaStream_t s);

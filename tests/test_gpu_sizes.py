@@ -1,6 +1,7 @@
-"""Grid sizes off the tuned list against the oracle: sizes whose strided tiles
-take several TMA boxes of narrow rows (each box must start on a 128-byte
-boundary of shared memory).
+"""Grid sizes off the tuned list: sizes whose strided tiles take several TMA
+boxes of narrow rows (each box must start on a 128-byte boundary of shared
+memory), and the size-specialised kernels with one tile shape, against the
+oracle and, where the oracle would take minutes, against the FP64 path.
 
 Tolerances as in test_gpu_parity: 1e-5 (FP32) and 1e-12 (FP64) relative L2.
 """
@@ -38,3 +39,30 @@ def check(gg, n, prec):
 @pytest.mark.parametrize("prec", ["f32", "f64"])
 def test_narrow_rows_in_several_boxes(gg, prec):
     check(gg, 324, prec)
+
+
+@pytest.mark.parametrize("n", [32, 48, 72, 96, 144, 216, 288])
+def test_one_shape_sizes_match_oracle(gg, n):
+    check(gg, n, "f32")
+
+
+@pytest.mark.parametrize("n", [432, 576, 648, 768, 864, 1024, 1152])
+def test_one_shape_sizes_match_fp64(gg, n):
+    ref = gg.Plan(n, float(n), BBKS, 50.0, "f64")
+    want = ref.zeldovich(seed=5, pos=False, vel=False)["psi"]
+    ref.sync()
+    ref.close()
+    plan = gg.Plan(n, float(n), BBKS, 50.0, "f32")
+    got = plan.zeldovich(seed=5, pos=True, vel=True)
+    plan.sync()
+    for layout in (False, True):
+        plan.set_layout(layout)
+        lay = plan.zeldovich(seed=5, psi=False)
+        plan.sync()
+        for j in range(3):
+            assert torch.equal(lay["vel"][j], got["vel"][j]), (layout, j)
+            assert torch.equal(lay["pos"][j], got["pos"][j]), (layout, j)
+    for j in range(3):
+        d = got["psi"][j].double() - want[j]
+        assert float(d.norm() / want[j].norm()) < 1e-5, j
+    plan.close()
