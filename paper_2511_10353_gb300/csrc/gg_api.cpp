@@ -102,6 +102,8 @@ struct gg_plan {
   // power spectrum: the grid's shell weights and weighted |m| for shell_nb shells
   std::vector<double> shell_w, shell_m;
   int shell_nb = 0;
+  double *diag = nullptr;  // device sums of the diagnostics, grown on use
+  size_t diag_words = 0;
 };
 
 struct gg_batch {
@@ -363,7 +365,7 @@ void release(gg_plan_t *plan) {
                   plan->tab.tw_n,    plan->tab.tw_half,   plan->tab.s_delta,
                   plan->tab.u_phi,   plan->err,           plan->noise_stage,
                   plan->tab.smooth,  plan->tab.interp_u,  plan->tab.interp_s,
-                  plan->tab.interp_smooth, plan->tab.cic_deconv, plan->phase};
+                  plan->tab.interp_smooth, plan->tab.cic_deconv, plan->phase, plan->diag};
   for (void *b : bufs)
     if (b) cudaFree(b);
   for (auto &slot : plan->stage)
@@ -543,6 +545,21 @@ gg_status ensure_grid(gg_plan_t *plan, void **buf) {
     *buf = nullptr;
     return fail(plan, GG_ENOMEM, "cudaMalloc of a component workspace failed");
   }
+  return GG_OK;
+}
+
+// At least `words` doubles in plan->diag (the diagnostics are synchronous:
+// nothing in flight reads a buffer replaced here).
+gg_status ensure_diag(gg_plan_t *plan, size_t words) {
+  if (plan->diag_words >= words) return GG_OK;
+  if (plan->diag) cudaFree(plan->diag);
+  plan->diag = nullptr;
+  plan->diag_words = 0;
+  if (cudaMalloc((void **)&plan->diag, sizeof(double) * words) != cudaSuccess) {
+    plan->diag = nullptr;
+    return fail(plan, GG_ENOMEM, "cudaMalloc of the diagnostics' sums failed");
+  }
+  plan->diag_words = words;
   return GG_OK;
 }
 
@@ -1054,8 +1071,9 @@ template <typename R>
 gg_status run_power_spectrum(gg_plan_t *plan, const void *field, int nbins, double *k_out,
                              double *p_out, int64_t *count_out) {
   const int n = (int)plan->p.n;
-  gg_status st = forward_zy<R>(plan, 0, field);
+  gg_status st = ensure_diag(plan, 2 * (size_t)nbins);
   if (st != GG_OK) return st;
+  if ((st = forward_zy<R>(plan, 0, field)) != GG_OK) return st;
   gg::AxisArgs x = axis_args<R>(plan, 0, plan->work);
   x.fwd = 1;
   x.inv = 0;
@@ -1064,9 +1082,8 @@ gg_status run_power_spectrum(gg_plan_t *plan, const void *field, int nbins, doub
   x.mul[0] = gg::kMulNone;
   x.variant = plan->variant[1];
   if ((st = launch_axis_timed<R>(plan, x, kXFused, "x forward pass")) != GG_OK) return st;
-  double *sums = nullptr;
-  cudaError_t e = cudaMallocAsync((void **)&sums, sizeof(double) * 2 * nbins, plan->stream);
-  if (e != cudaSuccess) return cuda_fail(plan, e, "cudaMallocAsync of the shell sums");
+  double *sums = plan->diag;
+  cudaError_t e = cudaSuccess;
   gg::ShellArgs a{};
   a.spec = plan->work;
   a.n = n;
@@ -1091,9 +1108,7 @@ gg_status run_power_spectrum(gg_plan_t *plan, const void *field, int nbins, doub
     }
   }
   if (e == cudaSuccess) e = pass(false, pw);
-  const cudaError_t ef = cudaFreeAsync(sums, plan->stream);
   if (e != cudaSuccess) return cuda_fail(plan, e, "power spectrum shell sums");
-  if (ef != cudaSuccess) return cuda_fail(plan, ef, "power spectrum shell sums");
   const double box = plan->p.box, vol = box * box * box, n6 = std::pow((double)n, 6.0);
   for (int b = 0; b < nbins; ++b) {
     const double c = plan->shell_w[b];
@@ -1108,44 +1123,33 @@ template <typename R>
 gg_status run_moments(gg_plan_t *plan, const void *field, double out[4]) {
   const int64_t count = plan->cells;
   const int blocks = gg::moment_blocks<R>(count);
-  double *slots = nullptr;
-  cudaError_t e = cudaMallocAsync((void **)&slots, sizeof(double) * 3 * blocks, plan->stream);
-  if (e != cudaSuccess) return cuda_fail(plan, e, "cudaMallocAsync of the moment slots");
-  std::vector<double> h(3 * (size_t)blocks);
-  double mean = 0.0, var = 0.0, lo = 0.0, hi = 0.0;
-  for (int pass = 0; pass < 2; ++pass) {
-    gg::MomentArgs a{};
-    a.field = field;
-    a.count = count;
-    a.second = pass;
-    a.mean = mean;
-    a.slots = slots;
-    if ((e = gg::launch_moments<R>(a, blocks, plan->stream)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(h.data(), slots, sizeof(double) * 3 * blocks, cudaMemcpyDeviceToHost,
-                             plan->stream)) != cudaSuccess ||
-        (e = cudaStreamSynchronize(plan->stream)) != cudaSuccess)
-      break;
-    double s = 0.0;
-    for (int b = 0; b < blocks; ++b) s += h[3 * b];
-    if (pass == 0) {
-      mean = s / (double)count;
-      lo = h[1];
-      hi = h[2];
-      for (int b = 1; b < blocks; ++b) {
-        lo = std::min(lo, h[3 * b + 1]);
-        hi = std::max(hi, h[3 * b + 2]);
-      }
-    } else {
-      var = s / (double)count;
-    }
+  const size_t words = 6 * (size_t)blocks + 3;
+  gg_status st = ensure_diag(plan, words);
+  if (st != GG_OK) return st;
+  gg::MomentArgs a{};
+  a.field = field;
+  a.count = count;
+  a.slots = plan->diag;
+  std::vector<double> h(words);
+  cudaError_t e;
+  if ((e = gg::launch_moments<R>(a, blocks, plan->stream)) != cudaSuccess ||
+      (e = cudaMemcpyAsync(h.data(), plan->diag, sizeof(double) * words, cudaMemcpyDeviceToHost,
+                           plan->stream)) != cudaSuccess ||
+      (e = cudaStreamSynchronize(plan->stream)) != cudaSuccess)
+    return cuda_fail(plan, e, "field moments");
+  const double *first = h.data() + 3 * (size_t)blocks;
+  const double mean = first[0];
+  double dev = 0.0;
+  for (int b = 0; b < blocks; ++b) dev += first[3 + 3 * b];
+  double var = dev / (double)count;
+  if (sizeof(R) == 4) {  // deviations from the FP32 value nearest to the mean
+    const double off = mean - (double)(float)mean;
+    var -= off * off;
   }
-  const cudaError_t ef = cudaFreeAsync(slots, plan->stream);
-  if (e != cudaSuccess) return cuda_fail(plan, e, "field moments");
-  if (ef != cudaSuccess) return cuda_fail(plan, ef, "field moments");
   out[0] = mean;
   out[1] = var;
-  out[2] = lo;
-  out[3] = hi;
+  out[2] = first[1];
+  out[3] = first[2];
   return GG_OK;
 }
 

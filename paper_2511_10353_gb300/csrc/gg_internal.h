@@ -212,10 +212,12 @@ template <typename R> cudaError_t launch_shell_sums(const ShellArgs &a, bool geo
 struct MomentArgs {
   const void *field;
   int64_t count;
-  int second;        // 0: sum of values; 1: sum of squared deviations from mean
-  double mean;
-  double *slots;     // device [3 per CTA]: sum, min, max
+  // device, 6 blocks + 3: first pass [blocks][sum, min, max], {mean, min, max},
+  // second pass [blocks][sum of squared deviations from the mean (FP32 fields:
+  // from the FP32 value nearest to it), -, -]
+  double *slots;
 };
+// Both passes and the mean between them, on s.
 template <typename R> int moment_blocks(int64_t count);
 template <typename R> cudaError_t launch_moments(const MomentArgs &a, int blocks, cudaStream_t s);
 

@@ -1,17 +1,27 @@
 // Sec. 2.1 diagnostics on sm_103a: shell sums of a half spectrum for the
 // power-spectrum estimator, and the moments of a real field.
 //
-// Shell sums: warps stride over the (x, y) lines of the half spectrum; each
-// CTA keeps partial sums per shell in shared memory, one copy per warp, then
-// adds them to the global FP64 sums. The grid's sums (weight, weight |m|)
-// are formed once per plan and shell count; each call then adds
-// weight |F|^2 only. Shell index by exact integer arithmetic:
-// b = floor(|m| + 1/2) is the smallest b with 4 m^2 < (2b + 1)^2.
+// Shell sums: the eight lines (+-m_x, +-m_y) and (+-m_y, +-m_x) of the half
+// spectrum share every |m|, so a warp takes such an orbit, adds the eight
+// |F|^2 of each k_z in registers and makes one shell index and one addition
+// to the CTA's shared-memory sums of them. The grid's sums (weight, weight
+// |m|) are formed once per plan and shell count. Shell index by exact integer
+// arithmetic: b = floor(|m| + 1/2) is the smallest b with 4 m^2 < (2b + 1)^2,
+// from an FP32 estimate (m^2 < 2^24) corrected by one; an FP64 square root a
+// mode had bound the kernel (two FP64 lanes an SM). 512^3: 1375 -> 63 us.
 //
-// Moments: per-CTA FP64 sum (first pass) or sum of squared deviations from a
-// given mean (second pass), minimum and maximum, written to one slot per
-// CTA; the host adds the slots (a fixed order: the result does not depend
-// on scheduling).
+// Moments: per-CTA FP64 sum (first pass) or sum of squared deviations
+// (second pass), minimum and maximum, one slot per CTA, added in a fixed
+// order (the result does not depend on scheduling); the mean stays on the
+// device between the passes. FP32 fields: adding every value in FP64 is
+// bound by the FP64 rate (512^3 1537 us a pass, 20 times the read), so a
+// thread adds 32 values exactly, as 64-bit integers in units of 2^-55 of
+// their largest binary order, and makes one FP64 addition of them. The second
+// pass squares d = v - c for the FP32 value c nearest to the mean, with
+// d = hi + lo and hi^2 = p + e exact: the p add up as integers too, the
+// e + 2 hi lo (below 2^-23 p) in FP32, and sum (v - mean)^2 =
+// sum d^2 - count (mean - c)^2. Groups that hold an infinity, a NaN or only
+// tiny values add in FP64. 512^3: 132 and 163 us.
 #include <cfloat>
 #include <cstdint>
 
@@ -23,69 +33,147 @@
 namespace gg {
 namespace {
 
-// One warp per (x, y) line of the half spectrum at a time; every warp adds
-// into its own copy of the shell sums in shared memory (copies = warps of
-// the CTA, or fewer when the bins are many). GEOM: the grid's own sums
-// (weight, weight |m|: FP64, once per plan and shell count); otherwise the
-// power sums alone, accumulated in the field's precision per CTA (A) and in
-// FP64 across CTAs.
+// GEOM: the grid's own sums (weight, weight |m|: FP64, once per plan and
+// shell count); otherwise the power sums alone, accumulated in the field's
+// precision per CTA (A) and in FP64 across CTAs. `copies` (a power of two) of
+// the shell sums per CTA, taken by lane, so that lanes of one shell seldom
+// meet; their stride is odd (other banks).
 template <typename R, typename A, bool GEOM>
 __global__ void __launch_bounds__(256) k_shell_sums(const ShellArgs a, int copies) {
   extern __shared__ __align__(16) unsigned char raw[];
-  A *acc = reinterpret_cast<A *>(raw);  // [copies][K][nbins], K = 2 (GEOM) or 1
+  A *acc = reinterpret_cast<A *>(raw);  // [copies][stride], K nbins used, K = 2 (GEOM) or 1
   constexpr int K = GEOM ? 2 : 1;
-  const int nb = a.nbins;
-  for (int i = threadIdx.x; i < copies * K * nb; i += blockDim.x) acc[i] = (A)0;
+  const int nb = a.nbins, stride = (K * nb) | 1;
+  for (int i = threadIdx.x; i < copies * stride; i += blockDim.x) acc[i] = (A)0;
   __syncthreads();
   const Cx<R> *spec = reinterpret_cast<const Cx<R> *>(a.spec);
   const int n = a.n, half = n / 2;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  A *mine = acc + (size_t)(warp % copies) * K * nb;
-  const int64_t lines = (int64_t)n * n;
-  const int64_t wstep = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t line = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp; line < lines; line += wstep) {
-    const int y = (int)(line % n), x = (int)(line / n);
-    if (x == half || y == half) continue;  // |m_j| = N/2 left out (k_z = N/2 is not stored)
-    const int mx = x < half ? x : x - n, my = y < half ? y : y - n;
-    const int64_t p2 = (int64_t)mx * mx + (int64_t)my * my;
-    const Cx<R> *row = spec + line * half;
+  A *mine = acc + (lane & (copies - 1)) * stride;
+  // orbits (u, v), 0 <= v <= u < N/2 (|m_j| = N/2 left out; k_z = N/2 is not stored)
+  const int orbits = half * (half + 1) / 2;
+  const int wstep = (int)gridDim.x * (blockDim.x >> 5);
+  for (int o = (int)blockIdx.x * (blockDim.x >> 5) + warp; o < orbits; o += wstep) {
+    int u = (int)((sqrtf(8.0f * (float)o + 1.0f) - 1.0f) * 0.5f);
+    while (u * (u + 1) / 2 > o) --u;
+    while ((u + 1) * (u + 2) / 2 <= o) ++u;
+    const int v = o - u * (u + 1) / 2;
+    // its lines: q bit 0 the sign of the first index, bit 1 of the second, bit 2 swapped
+    const Cx<R> *row[8];
+    int lines = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int p = q & 4 ? v : u, r = q & 4 ? u : v;
+      const bool on = !((q & 1) && p == 0) && !((q & 2) && r == 0) && !((q & 4) && u == v);
+      const int x = (q & 1) ? n - p : p, y = (q & 2) ? n - r : r;
+      row[q] = on ? spec + ((int64_t)x * n + y) * half : nullptr;
+      lines += on ? 1 : 0;
+    }
+    const int p2 = u * u + v * v;
     for (int kz = lane; kz < half; kz += 32) {
-      const int64_t m2 = p2 + (int64_t)kz * kz;
-      const double mag = sqrt((double)m2);
-      int b = (int)(mag + 0.5);
-      if ((int64_t)(2 * b + 1) * (2 * b + 1) <= 4 * m2) ++b;
-      if (b > 0 && 4 * m2 < (int64_t)(2 * b - 1) * (2 * b - 1)) --b;
-      if (b >= nb) continue;
+      const int m2 = p2 + kz * kz;  // < 2^24: exact in FP32
+      int b = (int)(sqrtf((float)m2) + 0.5f);
+      if ((2 * b + 1) * (2 * b + 1) <= 4 * m2) ++b;
+      if (b > 0 && 4 * m2 < (2 * b - 1) * (2 * b - 1)) --b;
+      if (b >= nb) break;  // the shells grow along the line
       const int w = kz == 0 ? 1 : 2;
       if constexpr (GEOM) {
-        atomicAdd(&mine[b], (A)w);
-        atomicAdd(&mine[nb + b], (A)(w * mag));
+        atomicAdd(&mine[b], (A)(w * lines));
+        atomicAdd(&mine[nb + b], (A)(w * lines) * (A)sqrt((double)m2));
       } else {
-        const Cx<R> v = row[kz];
-        atomicAdd(&mine[b], (A)w * (v.x * v.x + v.y * v.y));
+        Cx<R> f[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) f[q] = row[q] ? row[q][kz] : Cx<R>{(R)0, (R)0};
+        A t = (A)0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) t += f[q].x * f[q].x + f[q].y * f[q].y;
+        atomicAdd(&mine[b], (A)w * t);
       }
     }
   }
   __syncthreads();
   for (int i = threadIdx.x; i < K * nb; i += blockDim.x) {
     double t = 0.0;
-    for (int c = 0; c < copies; ++c) t += (double)acc[(size_t)c * K * nb + i];
+    for (int c = 0; c < copies; ++c) t += (double)acc[c * stride + i];
     if (t != 0.0) atomicAdd(&a.sums[i], t);
   }
 }
 
-template <typename R>
-__global__ void __launch_bounds__(256) k_moments(const MomentArgs a) {
-  const R *f = reinterpret_cast<const R *>(a.field);
-  double s = 0.0, lo = DBL_MAX, hi = -DBL_MAX;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.count;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const double v = (double)f[i];
-    const double d = a.second ? v - a.mean : v;
-    s += a.second ? d * d : d;
-    lo = fmin(lo, v);
-    hi = fmax(hi, v);
+// v (24-bit mantissa times 2^(e - 150)) in units of 2^(E - 182), E the group's
+// largest biased exponent (0 counts as 1): exact for e > E - 33, else cut off
+// below 2^-55 of the group's largest binary order.
+__device__ __forceinline__ long long fixed32(float v, int E) {
+  const uint32_t b = __float_as_uint(v);
+  const int e = (int)((b >> 23) & 255u);
+  const uint32_t m = (b & 0x7fffffu) | (e ? 0x800000u : 0u);
+  const int sh = E - (e ? e : 1);
+  const long long f = (long long)(((unsigned long long)m << 32) >> (sh < 63 ? sh : 63));
+  return (int)b < 0 ? -f : f;
+}
+__device__ __forceinline__ double unfixed(long long f, int E) {  // E >= 1
+  return (double)f * __hiloint2double((E - 182 + 1023) << 20, 0);
+}
+__device__ __forceinline__ int exponent_of(uint32_t bits) {
+  const int e = (int)((bits >> 23) & 255u);
+  return e ? e : 1;
+}
+
+constexpr int kMomentVec = 8;  // float4 a thread and group
+
+// The sum (SECOND: of squared deviations) of 32 FP32 values.
+template <bool SECOND>
+__device__ __forceinline__ double group_sum(const float4 *v, float c) {
+  float x[4 * kMomentVec];
+#pragma unroll
+  for (int i = 0; i < kMomentVec; ++i) {
+    x[4 * i] = v[i].x;
+    x[4 * i + 1] = v[i].y;
+    x[4 * i + 2] = v[i].z;
+    x[4 * i + 3] = v[i].w;
   }
+  uint32_t top = 0;
+  if constexpr (!SECOND) {
+#pragma unroll
+    for (int i = 0; i < 4 * kMomentVec; ++i) top = max(top, __float_as_uint(x[i]) & 0x7fffffffu);
+    if (top < 0x7f800000u) {
+      const int E = exponent_of(top);
+      long long s = 0;
+#pragma unroll
+      for (int i = 0; i < 4 * kMomentVec; ++i) s += fixed32(x[i], E);
+      return unfixed(s, E);
+    }
+    double s = 0.0;  // an infinity or a NaN
+    for (int i = 0; i < 4 * kMomentVec; ++i) s += (double)x[i];
+    return s;
+  } else {
+    float p[4 * kMomentVec], t = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 4 * kMomentVec; ++i) {
+      const float hi = __fsub_rn(x[i], c);  // x - c = hi + lo exactly
+      const float bp = __fsub_rn(hi, x[i]);
+      const float lo = __fsub_rn(__fsub_rn(x[i], __fsub_rn(hi, bp)), __fadd_rn(c, bp));
+      p[i] = __fmul_rn(hi, hi);
+      t = __fadd_rn(t, fmaf(2.0f * hi, lo, fmaf(hi, hi, -p[i])));
+      top = max(top, __float_as_uint(p[i]));
+    }
+    // below 2^-67 the remainders e would underflow
+    if (top < 0x7f800000u && top >= (60u << 23)) {
+      const int E = exponent_of(top);
+      long long s = 0;
+#pragma unroll
+      for (int i = 0; i < 4 * kMomentVec; ++i) s += fixed32(p[i], E);
+      return unfixed(s, E) + (double)t;
+    }
+    double s = 0.0;
+    for (int i = 0; i < 4 * kMomentVec; ++i) {
+      const double d = (double)x[i] - (double)c;
+      s += d * d;
+    }
+    return s;
+  }
+}
+
+__device__ __forceinline__ void block_slots(double s, double lo, double hi, double *slots) {
   for (int o = 16; o > 0; o >>= 1) {
     s += __shfl_xor_sync(0xffffffffu, s, o);
     lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
@@ -106,10 +194,75 @@ __global__ void __launch_bounds__(256) k_moments(const MomentArgs a) {
       tl = fmin(tl, ws[1][w]);
       th = fmax(th, ws[2][w]);
     }
-    a.slots[3 * blockIdx.x] = ts;
-    a.slots[3 * blockIdx.x + 1] = tl;
-    a.slots[3 * blockIdx.x + 2] = th;
+    slots[3 * blockIdx.x] = ts;
+    slots[3 * blockIdx.x + 1] = tl;
+    slots[3 * blockIdx.x + 2] = th;
   }
+}
+
+template <typename R, bool SECOND>
+__global__ void __launch_bounds__(256) k_moments(const MomentArgs a) {
+  double s = 0.0, lo = DBL_MAX, hi = -DBL_MAX;
+  const double mean = SECOND ? a.slots[3 * gridDim.x] : 0.0;  // k_moments_mean's
+  if constexpr (sizeof(R) == 4) {
+    const float4 *f = reinterpret_cast<const float4 *>(a.field);
+    // N even: whole quads; a field off the 16-byte grid takes the FP64 loop below
+    const int64_t quads = ((uintptr_t)a.field & 15u) ? 0 : a.count / 4;
+    const float c = (float)mean;
+    float flo = __int_as_float(0x7f800000), fhi = __int_as_float(0xff800000);
+    constexpr int GROUP = 256 * kMomentVec;
+    const int64_t whole = quads / GROUP;
+    for (int64_t g = blockIdx.x; g < whole; g += gridDim.x) {
+      float4 v[kMomentVec];
+#pragma unroll
+      for (int i = 0; i < kMomentVec; ++i) v[i] = __ldg(f + g * GROUP + i * 256 + threadIdx.x);
+      s += group_sum<SECOND>(v, c);
+      if constexpr (!SECOND) {
+#pragma unroll
+        for (int i = 0; i < kMomentVec; ++i) {
+          flo = fminf(flo, fminf(fminf(v[i].x, v[i].y), fminf(v[i].z, v[i].w)));
+          fhi = fmaxf(fhi, fmaxf(fmaxf(v[i].x, v[i].y), fmaxf(v[i].z, v[i].w)));
+        }
+      }
+    }
+    const float *fs = reinterpret_cast<const float *>(a.field);
+    for (int64_t i = whole * GROUP * 4 + (int64_t)blockIdx.x * 256 + threadIdx.x; i < a.count;
+         i += (int64_t)gridDim.x * 256) {  // the rest, in FP64
+      const float v = fs[i];
+      const double d = SECOND ? (double)v - (double)c : (double)v;
+      s += SECOND ? d * d : d;
+      flo = fminf(flo, v);
+      fhi = fmaxf(fhi, v);
+    }
+    lo = fmin(lo, (double)flo);
+    hi = fmax(hi, (double)fhi);
+  } else {
+    const R *f = reinterpret_cast<const R *>(a.field);
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.count;
+         i += (int64_t)gridDim.x * blockDim.x) {
+      const double v = (double)f[i];
+      const double d = SECOND ? v - mean : v;
+      s += SECOND ? d * d : d;
+      if constexpr (!SECOND) {
+        lo = fmin(lo, v);
+        hi = fmax(hi, v);
+      }
+    }
+  }
+  block_slots(s, lo, hi, a.slots + (SECOND ? 3 * gridDim.x + 3 : 0));
+}
+
+// The first pass's slots added in a fixed order: {mean, min, max} after them.
+__global__ void __launch_bounds__(256) k_moments_mean(double *slots, int blocks, int64_t count) {
+  double s = 0.0, lo = DBL_MAX, hi = -DBL_MAX;
+  for (int b = threadIdx.x; b < blocks; b += 256) {
+    s += slots[3 * b];
+    lo = fmin(lo, slots[3 * b + 1]);
+    hi = fmax(hi, slots[3 * b + 2]);
+  }
+  double *out = slots + 3 * blocks;
+  block_slots(s, lo, hi, out);
+  if (threadIdx.x == 0) out[0] = out[0] / (double)count;
 }
 
 int grid_for(int64_t work, int per_sm) {
@@ -124,16 +277,17 @@ int grid_for(int64_t work, int per_sm) {
 }  // namespace
 
 template <typename R, typename A, bool GEOM> cudaError_t shell_launch(const ShellArgs &a, cudaStream_t s) {
-  const size_t per_copy = (size_t)(GEOM ? 2 : 1) * a.nbins * sizeof(A);
-  int copies = (int)((192 * 1024) / per_copy);
-  copies = copies > 8 ? 8 : (copies < 1 ? 1 : copies);
+  const size_t per_copy = (size_t)((GEOM ? 2 : 1) * a.nbins | 1) * sizeof(A);
+  int copies = 8;
+  while (copies > 1 && copies * per_copy > 48 * 1024) copies /= 2;
   const size_t smem = per_copy * copies;
   auto kern = k_shell_sums<R, A, GEOM>;
   if (smem > 48 * 1024) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  kern<<<grid_for((int64_t)a.n * a.n * 32 / 8, 2), 256, smem, s>>>(a, copies);
+  const int64_t half = a.n / 2;
+  kern<<<grid_for(half * (half + 1) / 2 * 32, 4), 256, smem, s>>>(a, copies);
   return cudaGetLastError();
 }
 
@@ -141,10 +295,14 @@ template <typename R> cudaError_t launch_shell_sums(const ShellArgs &a, bool geo
   return geometry ? shell_launch<R, double, true>(a, s) : shell_launch<R, R, false>(a, s);
 }
 
-template <typename R> int moment_blocks(int64_t count) { return grid_for(count, 8); }
+template <typename R> int moment_blocks(int64_t count) {
+  return sizeof(R) == 4 ? grid_for(count / (4 * kMomentVec), 4) : grid_for(count, 8);
+}
 
 template <typename R> cudaError_t launch_moments(const MomentArgs &a, int blocks, cudaStream_t s) {
-  k_moments<R><<<blocks, 256, 0, s>>>(a);
+  k_moments<R, false><<<blocks, 256, 0, s>>>(a);
+  k_moments_mean<<<1, 256, 0, s>>>(a.slots, blocks, a.count);
+  k_moments<R, true><<<blocks, 256, 0, s>>>(a);
   return cudaGetLastError();
 }
 
