@@ -469,6 +469,7 @@ gg_status forward_zy(gg_plan_t *plan, uint64_t seed, const void *noise, void *ch
   z.tw_half = plan->tab.tw_half;
   z.tw_full = plan->tab.tw_n;
   z.variant = plan->variant[0];
+  z.err = plan->err;
   const double cb = (double)plan->cells * sizeof(R);
   cudaError_t e;
   {

@@ -675,6 +675,7 @@ template <typename R, int N, int V> struct ZPolicy {
   }
   static constexpr int MINB_INV = min_blocks(128 + DENSE * CB + WORK_INV * CB);
   static constexpr int MINB_FWD = min_blocks(WORK_FWD * CB);
+  static constexpr int MINB_NOISE = min_blocks(128 + DENSE * CB + WORK_FWD * CB);
 };
 
 }  // namespace ct

@@ -641,58 +641,89 @@ __global__ void __launch_bounds__(ct::ZPolicy<R, N, V>::THREADS, ct::ZPolicy<R, 
 // Forward z pass: Philox noise (or caller noise) of L lines into the padded
 // work tile, the length-N/2 transform in place, then the real-input unpacking
 // X_k = (Z_k + conj Z_{M-k})/2 - i/2 e^{-2 pi i k/N} (Z_k - conj Z_{M-k}).
-template <typename R, int N, int V>
-__device__ __forceinline__ void zfwd_body(const ZFwdArgs &a, int64_t t0, int64_t tstep,
+// NOISE: the caller's field, bulk-copied into a dense staging tile (as the
+// inverse pass does); the first stage reads it there, then the copy of the
+// CTA's next block starts and lands behind the remaining stages and the
+// stores. HBM-bound (8 B/cell); with per-thread loads, which nothing
+// overlapped, 512^3 took 245 us, now 181. Returns false when a copy
+// wait gave up.
+template <typename R, int N, int V, bool NOISE = false>
+__device__ __forceinline__ bool zfwd_body(const ZFwdArgs &a, int64_t t0, int64_t tstep,
                                           int64_t tlimit) {
   using C = Cx<R>;
   using Pol = ct::ZPolicy<R, N, V>;
   constexpr int M = Pol::M, E = Pol::E, P = Pol::P, L = Pol::L, LD = Pol::LD_FWD, PAD = Pol::PAD_FWD;
   constexpr int KM = ct::skey<R>(M);
   constexpr int S = ct::nstages(KM);
+  constexpr int DENSE_STRIDE = (int)(((Pol::DENSE * sizeof(C) + 127) / 128) * 128 / sizeof(C));
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  C *work = reinterpret_cast<C *>(smem_raw);
+  uint64_t *bar = reinterpret_cast<uint64_t *>(smem_raw);     // NOISE only
+  C *dense = reinterpret_cast<C *>(smem_raw + 128);           // NOISE only
+  C *work = NOISE ? dense + DENSE_STRIDE : reinterpret_cast<C *>(smem_raw);
   const int tid = threadIdx.x;
   const int64_t ntiles = a.nlines / L;
   const ct::Tw<C, false> tw_half{reinterpret_cast<const C *>(a.tw_half)};
   const C *twf = reinterpret_cast<const C *>(a.tw_full);
   if (tlimit > ntiles) tlimit = ntiles;
+  auto issue = [&](int64_t t) {
+    mbar_arrive_expect_tx(bar, (uint32_t)(Pol::DENSE * sizeof(C)));
+    bulk_load(dense, reinterpret_cast<const C *>(a.noise) + t * Pol::DENSE,
+              (uint32_t)(Pol::DENSE * sizeof(C)), bar);
+  };
+  if constexpr (NOISE) {
+    if (tid == 0) {
+      mbar_init(bar, 1);
+      fence_mbar_init();
+    }
+    __syncthreads();
+    if (tid == 0 && t0 < tlimit) issue(t0);
+  }
+  uint32_t phase = 0;
   for (int64_t t = t0; t < tlimit; t += tstep) {
     int l = tid / P, p = tid - (tid / P) * P;
     asm volatile("" : "+r"(l), "+r"(p));
     __builtin_assume(l >= 0 && l < L && p >= 0 && p < P);
     const int64_t line = t * L + l;
-    // line counts stay below 2^32 (N <= 4096, the host bounds the batch)
-    const uint32_t lpr = (uint32_t)(a.lines_per_real > 0 ? a.lines_per_real : a.nlines);
-    const uint32_t rr = (uint32_t)line / lpr, local = (uint32_t)line - rr * lpr;
-    static_assert(N % 4 == 0, "lines start on a Philox group");
-    const uint64_t g0 = (uint64_t)local * (uint64_t)(N / 4);
-    auto gen = [&](uint64_t seed) {
-#pragma unroll
-      for (int i = 0; i < E / 2; ++i) {
-        const int q = p + P * i;
-        R w[4];
-        if constexpr ((int64_t)N * N * N / 4 <= 0xFFFFFFFFll)  // group indices fit 32 bits
-          gauss4(noise_words32(seed, (uint32_t)(g0 + q)), w);
-        else
-          gauss4(noise_words(seed, g0 + q), w);
-        work[zpad<LD, PAD>(l, 2 * q)] = C{w[0], w[1]};
-        work[zpad<LD, PAD>(l, 2 * q + 1)] = C{w[2], w[3]};
-      }
-    };
-    if (a.noise) {
-      const C *src = reinterpret_cast<const C *>(a.noise) + line * M;
-#pragma unroll
-      for (int i = 0; i < E; ++i) work[zpad<LD, PAD>(l, p + P * i)] = src[p + P * i];
-    } else if (!a.seeds) {  // one seed for the launch: its key schedule is uniform
-      gen(a.seed);
-    } else {
-      gen(a.seeds[rr]);
-    }
-    ct::stage_barrier<Pol::SY>();
     auto ld_w = [&](int n) { return work[zpad<LD, PAD>(l, n)]; };
     auto st_w = [&](int n, C v) { work[zpad<LD, PAD>(l, n)] = v; };
+    constexpr int FIRST = NOISE ? 1 : 0;  // the stage the work tile's transform starts at
+    if constexpr (NOISE) {
+      const bool ok = __syncthreads_and(mbar_wait(bar, phase, a.err));
+      if (!ok) return false;  // nothing else in flight: the next copy is issued after this wait
+      phase ^= 1;
+      const C *dl = dense + l * M;
+      auto ld_d = [&](int n) { return dl[n]; };
+      ct::stage<R, M, E, 0, false, ct::kSyncNone>(p, tw_half, ld_d, st_w);
+      __syncthreads();
+      if (tid == 0 && t + tstep < tlimit) {  // the dense tile has been read: fetch the next block
+        fence_proxy_async_smem();
+        issue(t + tstep);
+      }
+    } else {
+      // line counts stay below 2^32 (N <= 4096, the host bounds the batch)
+      const uint32_t lpr = (uint32_t)(a.lines_per_real > 0 ? a.lines_per_real : a.nlines);
+      const uint32_t rr = (uint32_t)line / lpr, local = (uint32_t)line - rr * lpr;
+      static_assert(N % 4 == 0, "lines start on a Philox group");
+      const uint64_t g0 = (uint64_t)local * (uint64_t)(N / 4);
+      auto gen = [&](uint64_t seed) {
+#pragma unroll
+        for (int i = 0; i < E / 2; ++i) {
+          const int q = p + P * i;
+          R w[4];
+          if constexpr ((int64_t)N * N * N / 4 <= 0xFFFFFFFFll)  // group indices fit 32 bits
+            gauss4(noise_words32(seed, (uint32_t)(g0 + q)), w);
+          else
+            gauss4(noise_words(seed, g0 + q), w);
+          st_w(2 * q, C{w[0], w[1]});
+          st_w(2 * q + 1, C{w[2], w[3]});
+        }
+      };
+      if (!a.seeds) gen(a.seed);  // one seed for the launch: its key schedule is uniform
+      else gen(a.seeds[rr]);
+      ct::stage_barrier<Pol::SY>();
+    }
     if constexpr (Pol::FUSE) {  // the last two stages in registers, stored in natural order
-      ct::stages<R, M, E, false, 0, S - 2, Pol::SY>(p, tw_half, ld_w, st_w);
+      ct::stages<R, M, E, false, FIRST, S - 2, Pol::SY>(p, tw_half, ld_w, st_w);
       constexpr int RB = ct::radix_of(KM, S - 1, false), NBB = E / RB, SPANB = M / RB;
       C v[E];
       ct::last_two_stages_regs<R, M, E>(p, tw_half, ld_w, v);
@@ -703,7 +734,7 @@ __device__ __forceinline__ void zfwd_body(const ZFwdArgs &a, int64_t t0, int64_t
         for (int r = 0; r < RB; ++r) st_w(p + P * b + r * SPANB, v[b * RB + r]);
       ct::stage_barrier<Pol::SY>();
     } else {
-      ct::stages<R, M, E, false, 0, S, Pol::SY>(p, tw_half, ld_w, st_w);
+      ct::stages<R, M, E, false, FIRST, S, Pol::SY>(p, tw_half, ld_w, st_w);
     }
     // X_k = S/2 + D u_k with S = Z_k + conj Z_{M-k}, D = Z_k - conj Z_{M-k},
     // u_k = -(i/2) w_k; the partner X_{M-k} = conj(S/2 - D u_k) (w_{M-k} =
@@ -733,12 +764,14 @@ __device__ __forceinline__ void zfwd_body(const ZFwdArgs &a, int64_t t0, int64_t
     }
     ct::stage_barrier<Pol::SY>();  // the work tile's lines are rewritten next tile
   }
+  return true;
 }
 
-template <typename R, int N, int V>
-__global__ void __launch_bounds__(ct::ZPolicy<R, N, V>::THREADS, ct::ZPolicy<R, N, V>::MINB_FWD)
+template <typename R, int N, int V, bool NOISE>
+__global__ void __launch_bounds__(ct::ZPolicy<R, N, V>::THREADS,
+                                  NOISE ? ct::ZPolicy<R, N, V>::MINB_NOISE : ct::ZPolicy<R, N, V>::MINB_FWD)
     k_zfwd_ct(const ZFwdArgs a) {
-  zfwd_body<R, N, V>(a, blockIdx.x, gridDim.x, INT64_MAX);
+  zfwd_body<R, N, V, NOISE>(a, blockIdx.x, gridDim.x, INT64_MAX);
 }
 
 // ------------------------------------------------------------ launchers
@@ -795,11 +828,12 @@ cudaError_t ct_launch_zinv(const ZInvArgs &a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-template <typename R, int N, int V>
+template <typename R, int N, int V, bool NOISE>
 cudaError_t ct_launch_zfwd(const ZFwdArgs &a, cudaStream_t s) {
   using Pol = ct::ZPolicy<R, N, V>;
-  const size_t smem = (size_t)Pol::WORK_FWD * 2 * sizeof(R);
-  auto kern = k_zfwd_ct<R, N, V>;
+  const size_t dense = (Pol::DENSE * 2 * sizeof(R) + 127) & ~(size_t)127;
+  const size_t smem = (NOISE ? 128 + dense : 0) + (size_t)Pol::WORK_FWD * 2 * sizeof(R);
+  auto kern = k_zfwd_ct<R, N, V, NOISE>;
   cudaError_t e = set_smem(kern, smem);
   if (e != cudaSuccess) return e;
   kern<<<persistent_blocks(kern, Pol::THREADS, smem, a.nlines / Pol::L), Pol::THREADS, smem, s>>>(a);
@@ -877,13 +911,16 @@ template <typename R, int... NS> struct CtTable {
     }
     return zinv_v<N, 0>(a, s);
   }
+  template <int N, int V> static cudaError_t zfwd_v(const ZFwdArgs &a, cudaStream_t s) {
+    return a.noise ? ct_launch_zfwd<R, N, V, true>(a, s) : ct_launch_zfwd<R, N, V, false>(a, s);
+  }
   template <int N> static cudaError_t zfwd_n(const ZFwdArgs &a, cudaStream_t s) {
     if constexpr (ct::ct_tuned<R>(N)) {
-      if (a.variant == 1) return ct_launch_zfwd<R, N, 1>(a, s);
-      if (a.variant == 2) return ct_launch_zfwd<R, N, 2>(a, s);
-      if (a.variant == 3) return ct_launch_zfwd<R, N, 3>(a, s);
+      if (a.variant == 1) return zfwd_v<N, 1>(a, s);
+      if (a.variant == 2) return zfwd_v<N, 2>(a, s);
+      if (a.variant == 3) return zfwd_v<N, 3>(a, s);
     }
-    return ct_launch_zfwd<R, N, 0>(a, s);
+    return zfwd_v<N, 0>(a, s);
   }
   static cudaError_t zinv(const ZInvArgs &a, cudaStream_t s) {
     cudaError_t e = cudaErrorInvalidValue;

@@ -116,6 +116,7 @@ struct ZFwdArgs {
   int variant;            // tile variant of the size-specialised kernel
   const uint64_t *seeds;  // batched form: device array, one seed per realization (else seed)
   int64_t lines_per_real; // lines of one realization (<= 0: nlines)
+  int *err;               // device error word (caller noise: a copy wait gave up)
 };
 
 // Inverse z pass (c2r) with the Zel'dovich epilogue (Eq. 3) or a plain real

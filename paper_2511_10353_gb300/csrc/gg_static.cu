@@ -129,6 +129,7 @@ gg_status run(const gg_params *p, const gg_info &info, const double *sd, uint64_
   z.st = st_half;
   z.tw_half = s.tw_half;
   z.tw_full = s.tw_n;
+  z.err = s.err;
   const int lines = gg::z_lines_per_cta<R>(st_half);  // the rule gg_plan uses
   z.lines_per_cta = lines;
   e = spec ? gg::spec_zfwd<R>(z, st) : gg::launch_zfwd<R>(z, st);
