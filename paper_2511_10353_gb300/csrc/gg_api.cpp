@@ -68,7 +68,7 @@ struct gg_plan {
   // 0 z forward, 1 y forward, 2 x fused, 3 y inverse (x branch),
   // 4 y inverse (y/z branches), 5 z inverse
   int variant[6] = {0, 0, 0, 0, 0, 0};
-  int chunked = 0;  // 1: the three-component chain keeps the spectrum chunk-major
+  int chunked = 0;  // 1: the three-component chain keeps the spectrum chunk-major (gg_plan_set_layout)
   // fault test (gg_test_arm_fault): the next y forward pass issues no copies
   int test_skip_copy = 0;
   uint32_t test_wait_us = 0;
@@ -453,14 +453,13 @@ gg_status launch_axis_timed(gg_plan_t *plan, const gg::AxisArgs &c, int kind, co
   return e == cudaSuccess ? GG_OK : cuda_fail(plan, e, what);
 }
 
-// z forward (noise or caller noise) and y forward into plan->work.
+// z forward (noise or caller noise) into dst.
 template <typename R>
-gg_status forward_zy(gg_plan_t *plan, uint64_t seed, const void *noise, void *chunked_dst = nullptr,
-                     int chunk_b = 0) {
+gg_status forward_z(gg_plan_t *plan, uint64_t seed, const void *noise, void *dst) {
   const int n = (int)plan->p.n;
   gg::ZFwdArgs z{};
   z.noise = noise;
-  z.out = plan->work;
+  z.out = dst;
   z.seed = seed;
   z.nlines = (int64_t)n * n;
   z.n = n;
@@ -476,7 +475,15 @@ gg_status forward_zy(gg_plan_t *plan, uint64_t seed, const void *noise, void *ch
     ProfScope ps(plan, kZFwd, noise ? 2 * cb : cb);
     e = gg::spec_has<R>(n) ? gg::spec_zfwd<R>(z, plan->stream) : gg::launch_zfwd<R>(z, plan->stream);
   }
-  if (e != cudaSuccess) return cuda_fail(plan, e, "z forward pass");
+  return e == cudaSuccess ? GG_OK : cuda_fail(plan, e, "z forward pass");
+}
+
+// z forward (noise or caller noise) and y forward into plan->work.
+template <typename R>
+gg_status forward_zy(gg_plan_t *plan, uint64_t seed, const void *noise, void *chunked_dst = nullptr,
+                     int chunk_b = 0) {
+  const gg_status st = forward_z<R>(plan, seed, noise, plan->work);
+  if (st != GG_OK) return st;
   gg::AxisArgs c = axis_args<R>(plan, 1, plan->work);
   c.fwd = 1;
   c.inv = 0;
@@ -965,11 +972,72 @@ gg_status autotune(gg_plan_t *plan, int reps) {
 // ------------------------------------------------------------ adjoint form
 // psi_j = J_j W with J_j = F^-1 diag(i m_j U) F (F the unnormalised DFT,
 // U real and even in k). i m_j U is purely imaginary and Hermitian, so
-// J_j^T = -J_j and dL/dW = sum_j J_j^T g_j = -sum_j J_j g_j: the forward
-// chain run once per component on g_j, accumulated with weight -1. No
-// transform intermediates are stored.
+// J_j^T = -J_j and dL/dW = sum_j J_j^T g_j = -sum_j J_j g_j. No transform
+// intermediates are stored.
+//
+// All three gradients: the transpose of the forward schedule, their spectra
+// joined where a factor commutes with the transforms left (72 B/cell):
+//   z forward g_x -> work, g_y -> work2, g_z -> g_noise
+//   y forward work; (work2, g_noise) -> work2 = i m_y Y[.] + i m_z Y[.]
+//   x fused   (work, work2) -> work = X^-1[-U (i m_x X[.] + X[.])]
+//   y inverse, z inverse -> g_noise
+// 512^3: 3.45 ms as one chain per component (128 B/cell), now 1.73.
+template <typename R>
+gg_status run_adjoint3(gg_plan_t *plan, const void *const g_psi[3], void *g_noise) {
+  gg_status st;
+  void *const half[3] = {plan->work, plan->work2, g_noise};
+  for (int j = 0; j < 3; ++j)
+    if ((st = forward_z<R>(plan, 0, g_psi[j], half[j])) != GG_OK) return st;
+  const double cb = (double)plan->cells * sizeof(R);
+  cudaError_t e;
+  gg::AxisArgs y = axis_args<R>(plan, 1, plan->work);
+  y.fwd = 1;
+  y.nout = 1;
+  y.dst[0] = plan->work;
+  y.variant = plan->variant[1];
+  if ((st = launch_axis_timed<R>(plan, y, kYFwd, "y forward pass")) != GG_OK) return st;
+  gg::AxisArgs d = axis_args<R>(plan, 1, plan->work2);
+  d.src2 = g_noise;
+  d.fwd = 1;
+  d.nout = 1;
+  d.dst[0] = plan->work2;
+  {
+    ProfScope ps(plan, kYFwd, 3 * cb);
+    e = gg::spec_axis_dual<R>(d, plan->stream);
+  }
+  if (e != cudaSuccess) return cuda_fail(plan, e, "y forward pass (two inputs)");
+  gg::AxisArgs x = axis_args<R>(plan, 0, plan->work);
+  x.src2 = plan->work2;
+  x.fwd = 1;
+  x.inv = 1;
+  x.pre = 1;
+  x.table = plan->tab.u_phi;
+  x.interp = plan->tab.interp_u;
+  x.interp_cells = plan->tab.interp_cells;
+  x.nout = 1;
+  x.dst[0] = plan->work;
+  {
+    ProfScope ps(plan, kXFused, 3 * cb);
+    e = gg::spec_axis_dual<R>(x, plan->stream);
+  }
+  if (e != cudaSuccess) return cuda_fail(plan, e, "x fused pass (two inputs)");
+  gg::AxisArgs yi = axis_args<R>(plan, 1, plan->work);
+  yi.inv = 1;
+  yi.nout = 1;
+  yi.dst[0] = plan->work;
+  yi.variant = plan->variant[3];
+  if ((st = launch_axis_timed<R>(plan, yi, kYInvX, "y inverse pass")) != GG_OK) return st;
+  return zinv_pass<R>(plan, 0, plan->work, g_noise, nullptr, nullptr, false);
+}
+
+// Some gradients only, or a size without specialised kernels: the forward
+// chain once per component, accumulated with weight -1.
 template <typename R>
 gg_status run_adjoint(gg_plan_t *plan, const void *const g_psi[3], void *g_noise) {
+  if (g_psi && g_psi[0] && g_psi[1] && g_psi[2] && gg::spec_has<R>((int)plan->p.n)) {
+    const gg_status st = ensure_grid(plan, &plan->work2);
+    return st != GG_OK ? st : run_adjoint3<R>(plan, g_psi, g_noise);
+  }
   cudaError_t e = cudaMemsetAsync(g_noise, 0, (size_t)plan->cells * sizeof(R), plan->stream);
   if (e != cudaSuccess) return cuda_fail(plan, e, "cudaMemsetAsync");
   for (int j = 0; j < 3; ++j) {

@@ -427,6 +427,202 @@ __global__ void __launch_bounds__(ct::AxisPolicy<R, N, V>::THREADS, ct::AxisPoli
   axis_body<R, N, V, MODE, CUT, FILT>(map, a, blockIdx.x, gridDim.x, INT64_MAX, &smap0, &smap1);
 }
 
+// Two inputs, one output: the transpose of the two-output passes (the adjoint
+// of Eqs. 1-2). DUAL = kDualY, forward y only: X = i m_y Y[src] + i m_z Y[src2]
+// to dst[0]; kDualX, forward x, filter (a.interp or a.table) and inverse:
+// X^-1[-U (i m_x X[src] + X[src2])] to dst[0]. The first input's spectrum,
+// times its factor, is parked in its own tile buffer (each thread reads back
+// what it wrote); the second buffer then holds the work tile, from which the
+// output leaves by TMA. The next tile's first copy starts once the parked
+// spectrum has been read, its second once the output store has read the tile.
+// 512^3: y 251 us, x 425 us (12 B/cell each; bound by issue like the other
+// strided passes; 288 and 523 us with one 256-thread CTA an SM).
+constexpr int kDualY = 1, kDualX = 2;
+// the tile shape: variant 2 where it puts three CTAs on an SM
+template <typename R, int N>
+using DualPolicy = ct::AxisPolicy<R, N, ct::AxisPolicy<R, N, 2>::THREE ? 2 : 0>;
+template <typename R, int N, int DUAL>
+__global__ void __launch_bounds__(DualPolicy<R, N>::THREADS, DualPolicy<R, N>::MINB)
+    k_axis_dual(const __grid_constant__ CUtensorMap map0, const __grid_constant__ CUtensorMap map1,
+                const __grid_constant__ CUtensorMap smap, const AxisArgs a) {
+  using C = Cx<R>;
+  using Pol = DualPolicy<R, N>;
+  constexpr int K = ct::skey<R>(N);
+  constexpr int B = Pol::B, E = Pol::E, P = Pol::P, HALF = N / 2, S = ct::nstages(K);
+  constexpr int TILE = N * B, INNER = HALF / B;
+  constexpr int TILE_STRIDE = (int)(((TILE * sizeof(C) + 127) / 128) * 128 / sizeof(C));
+  constexpr int RH = ct::radix_of(K, 0, true), SPAN = N / RH, NB = E / RH;
+  constexpr bool FUSE = ct::fuse_pair<R, N, E>();
+  static_assert(S > 1, "in-place last stage");
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  uint64_t *bars = reinterpret_cast<uint64_t *>(smem_raw);
+  C *bufs = reinterpret_cast<C *>(smem_raw + 128);
+  float *f_exact = reinterpret_cast<float *>(bufs + 2 * TILE_STRIDE);
+  float4 *f_cells = reinterpret_cast<float4 *>(f_exact + kInterpExact);
+  const int tid = threadIdx.x;
+  const int64_t ntiles = (int64_t)N * INNER;
+  const R *table = reinterpret_cast<const R *>(a.table);
+  const bool interp = DUAL == kDualX && sizeof(R) == 4 && a.interp;
+  constexpr bool TW_SMEM = Pol::TW_SMEM;
+  C *tw_s = bufs + 2 * TILE_STRIDE + (interp ? (kInterpExact + 4 * kMaxInterpCells(N)) / 2 : 0);
+  if constexpr (TW_SMEM) {
+    const C *src = reinterpret_cast<const C *>(a.tw);
+    for (int i = tid; i < N; i += blockDim.x) tw_s[i] = src[i];
+  }
+  const ct::Tw<C, TW_SMEM> tw{TW_SMEM ? tw_s : reinterpret_cast<const C *>(a.tw)};
+  if (interp) {
+    const float *src = reinterpret_cast<const float *>(a.interp);
+    for (int i = tid; i < kInterpExact; i += blockDim.x) f_exact[i] = src[i];
+    const float4 *cs = reinterpret_cast<const float4 *>(src + kInterpExact);
+    for (int i = tid; i < a.interp_cells; i += blockDim.x) f_cells[i] = cs[i];
+  }
+  if (tid == 0) {
+    mbar_init(&bars[0], 1);
+    mbar_init(&bars[1], 1);
+    fence_mbar_init();
+  }
+  __syncthreads();
+  auto issue = [&](int64_t t, int part) {
+    const int outer = (int)(t / INNER), chunk = (int)(t - (int64_t)outer * INNER);
+    const CUtensorMap *map = part ? &map1 : &map0;
+    C *dst = bufs + part * TILE_STRIDE;
+    mbar_arrive_expect_tx(&bars[part], (uint32_t)(TILE * sizeof(C)));
+#pragma unroll
+    for (int i = 0; i < N; i += Pol::ROWS_BOX) {
+      if (DUAL == kDualY) tma_load_4d(dst + i * B, map, &bars[part], chunk * B * 2, i, outer, 0);
+      else tma_load_4d(dst + i * B, map, &bars[part], chunk * B * 2, outer, i, 0);
+    }
+  };
+  int64_t t = blockIdx.x;
+  if (tid == 0 && t < ntiles) {
+    issue(t, 0);
+    issue(t, 1);
+  }
+  uint32_t phase = 0;
+  C *b0 = bufs, *b1 = bufs + TILE_STRIDE;
+  for (; t < ntiles; t += gridDim.x, phase ^= 1) {
+    const int64_t tn = t + gridDim.x;
+    int c = tid & (B - 1), p = tid / B;
+    asm volatile("" : "+r"(c), "+r"(p));
+    __builtin_assume(c >= 0 && c < B && p >= 0 && p < P);
+    const int outer = (int)(t / INNER), chunk = (int)(t - (int64_t)outer * INNER);
+    const int kz = chunk * B + c;
+    auto forward = [&](C *buf, C *X) {
+      auto ld = [&](int n) { return buf[n * B + c]; };
+      auto st = [&](int n, C v) { buf[n * B + c] = v; };
+      if constexpr (FUSE) {
+        ct::stages<R, N, E, false, 0, S - 2>(p, tw, ld, st);
+        ct::last_two_stages_regs<R, N, E>(p, tw, ld, X);
+      } else {
+        ct::stages<R, N, E, false, 0, S - 1>(p, tw, ld, st);
+        ct::last_stage_regs<R, N, E, false>(p, tw, ld, X);
+      }
+    };
+    C X[E];
+    bool ok = __syncthreads_and(mbar_wait(&bars[0], phase, a.err, a.wait_us));
+    if (!ok) {  // the tile's second copy may be in flight
+      if (tid == 0) {
+        mbar_wait(&bars[1], phase, nullptr, a.wait_us);
+        bulk_wait0();
+      }
+      return;
+    }
+    forward(b0, X);
+    __syncthreads();  // every thread has read the tile
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+#pragma unroll
+      for (int r = 0; r < RH; ++r) {
+        const int n = p + P * b + r * SPAN;
+        const R f = n == HALF ? (R)0 : (R)ct_freq(n, N);
+        const C v = X[b * RH + r];
+        b0[n * B + c] = C{-f * v.y, f * v.x};
+      }
+    ok = __syncthreads_and(mbar_wait(&bars[1], phase, a.err, a.wait_us));
+    if (!ok) {  // no other copy in flight
+      if (tid == 0) bulk_wait0();
+      return;
+    }
+    forward(b1, X);
+    const int m_outer = DUAL == kDualX ? ct_freq(outer, N) : 0;
+    const bool nyq_outer = DUAL == kDualX && outer == HALF;
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+#pragma unroll
+      for (int r = 0; r < RH; ++r) {
+        const int n = p + P * b + r * SPAN;
+        const C u = b0[n * B + c], v = X[b * RH + r];
+        if constexpr (DUAL == kDualY) {
+          X[b * RH + r] = C{u.x - (R)kz * v.y, u.y + (R)kz * v.x};
+        } else {
+          const int m = ct_freq(n, N);
+          const int q = (n == HALF || nyq_outer) ? -1 : m * m + m_outer * m_outer + kz * kz;
+          R f;
+          if (q < 0) {
+            f = (R)0;
+          } else if (!interp) {
+            f = __ldg(table + q);
+          } else if (q < kInterpExact) {
+            f = (R)f_exact[q];
+          } else {  // cubic Hermite in m = sqrt(m2), unit cells, Horner form
+            const float mf = (float)q;
+            const float mm = mf * rsqrtf(mf);
+            const int j = (int)mm;
+            const float d = mm - (float)j;
+            const float4 cc = f_cells[j - kInterpFirstCell];
+            f = (R)fmaf(d, fmaf(d, fmaf(d, cc.w, cc.z), cc.y), cc.x);
+          }
+          X[b * RH + r] = C{-f * (u.x + v.x), -f * (u.y + v.y)};
+        }
+      }
+    __syncthreads();  // both tiles have been read
+    if (tid == 0 && tn < ntiles) {
+      fence_proxy_async_smem();
+      issue(tn, 0);
+    }
+    auto ld = [&](int n) { return b1[n * B + c]; };
+    auto st = [&](int n, C v) { b1[n * B + c] = v; };
+    if constexpr (DUAL == kDualY) {
+#pragma unroll
+      for (int b = 0; b < NB; ++b)
+#pragma unroll
+        for (int r = 0; r < RH; ++r) st(p + P * b + r * SPAN, X[b * RH + r]);
+      fence_proxy_async_smem();
+      __syncthreads();
+    } else if constexpr (FUSE) {
+      ct::inverse_head_regs<R, N, E>(tw, X);
+      ct::inverse_head_store<R, N, E>(p, X, st);
+      __syncthreads();
+      ct::stages<R, N, E, true, 2, S - 1>(p, tw, ld, st);
+      ct::stage<R, N, E, S - 1, true, ct::kSyncCtaAsync>(p, tw, ld, st);
+    } else {
+#pragma unroll
+      for (int b = 0; b < NB; ++b) Butterfly<RH, true, C>::run(&X[b * RH]);
+#pragma unroll
+      for (int b = 0; b < NB; ++b)
+#pragma unroll
+        for (int r = 0; r < RH; ++r) st((p + P * b) * RH + r, X[b * RH + r]);
+      __syncthreads();
+      ct::stages<R, N, E, true, 1, S - 1>(p, tw, ld, st);
+      ct::stage<R, N, E, S - 1, true, ct::kSyncCtaAsync>(p, tw, ld, st);
+    }
+    if (tid == 0) {
+#pragma unroll
+      for (int i = 0; i < N; i += Pol::ROWS_BOX) {
+        if (DUAL == kDualY) tma_store_4d(&smap, b1 + i * B, chunk * B * 2, i, outer, 0);
+        else tma_store_4d(&smap, b1 + i * B, chunk * B * 2, outer, i, 0);
+      }
+      bulk_commit();
+      if (tn < ntiles) {
+        bulk_wait_read0();
+        fence_proxy_async_smem();
+        issue(tn, 1);
+      }
+    }
+  }
+  if (tid == 0) bulk_wait0();  // the output stores, before the CTA exits
+}
+
 // ------------------------------------------------------------ z passes
 // Padded line layout of the z-pass work tile: element n of line l at
 // l * LD + n + n / PAD (PAD a power of two or 0: no padding; pairs
@@ -816,6 +1012,35 @@ cudaError_t ct_launch_axis(const AxisArgs &in, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+template <typename R, int N, int DUAL>
+cudaError_t ct_launch_dual(const AxisArgs &in, cudaStream_t s) {
+  using Pol = DualPolicy<R, N>;
+  AxisArgs a = in;
+  a.axis = DUAL == kDualY ? 1 : 0;
+  a.cols = Pol::B;
+  a.rows_box = Pol::ROWS_BOX;
+  a.chunked_in = a.chunked_out = a.nbatch = 0;
+  CUtensorMap map[3];
+  const void *bufs[3] = {a.src, a.src2, a.dst[0]};
+  cudaError_t e;
+  for (int i = 0; i < 3; ++i) {
+    AxisArgs b = a;
+    b.src = bufs[i];
+    if ((e = make_map<R>(&map[i], b)) != cudaSuccess) return e;
+  }
+  const size_t tile = ((size_t)N * Pol::B * 2 * sizeof(R) + 127) & ~(size_t)127;
+  const bool interp = DUAL == kDualX && sizeof(R) == 4 && a.interp;
+  if (interp && a.interp_cells > kMaxInterpCells(N)) return cudaErrorInvalidValue;
+  const int cells = Pol::TW_SMEM ? kMaxInterpCells(N) : a.interp_cells;  // as ct_launch_axis
+  const size_t smem = 128 + 2 * tile + (interp ? kInterpExact * sizeof(float) + (size_t)cells * 16 : 0) +
+                      (Pol::TW_SMEM ? (size_t)N * 2 * sizeof(R) : 0);
+  auto kern = k_axis_dual<R, N, DUAL>;
+  if ((e = set_smem(kern, smem)) != cudaSuccess) return e;
+  const int64_t tiles = (int64_t)N * ((N / 2) / Pol::B);
+  kern<<<persistent_blocks(kern, Pol::THREADS, smem, tiles), Pol::THREADS, smem, s>>>(map[0], map[1], map[2], a);
+  return cudaGetLastError();
+}
+
 template <typename R, int N, int V, bool EXT = false, int OUT = 0>
 cudaError_t ct_launch_zinv(const ZInvArgs &a, cudaStream_t s) {
   using Pol = ct::ZPolicy<R, N, V>;
@@ -884,6 +1109,12 @@ template <typename R, int... NS> struct CtTable {
   static cudaError_t axis(const AxisArgs &a, cudaStream_t s) {
     cudaError_t e = cudaErrorInvalidValue;
     ((a.n == NS ? (e = axis_n<NS>(a, s), 0) : 0), ...);
+    return e;
+  }
+  // two inputs, one output: a.inv 0 the y pass, 1 the x pass (see k_axis_dual)
+  static cudaError_t dual(const AxisArgs &a, cudaStream_t s) {
+    cudaError_t e = cudaErrorInvalidValue;
+    ((a.n == NS ? (e = a.inv ? ct_launch_dual<R, NS, kDualX>(a, s) : ct_launch_dual<R, NS, kDualY>(a, s), 0) : 0), ...);
     return e;
   }
   template <int N, int V> static cudaError_t zinv_v(const ZInvArgs &a, cudaStream_t s) {

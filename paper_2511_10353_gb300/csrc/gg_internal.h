@@ -61,6 +61,7 @@ enum Mul : int {
 //  !fwd &&  inv : for each output o: x mul[o], inverse transform -> dst[o]
 struct AxisArgs {
   const void *src;
+  const void *src2;       // the two-input passes (spec_axis_dual) only
   void *dst[3];
   int nout;
   int mul[3];
@@ -243,11 +244,16 @@ template <typename R> bool spec_tuned(int n);  // has tile variants (gg_autotune
 bool spec_more_has_f32(int n);
 int spec_more_cols_f32(int n, int v);
 cudaError_t spec_more_axis_f32(const AxisArgs &a, cudaStream_t s);
+cudaError_t spec_more_dual_f32(const AxisArgs &a, cudaStream_t s);
 cudaError_t spec_more_zinv_f32(const ZInvArgs &a, cudaStream_t s);
 cudaError_t spec_more_zfwd_f32(const ZFwdArgs &a, cudaStream_t s);
 constexpr int kSpecAxisVariants = 3;  // tile variants the autotuner times per strided pass
 constexpr int kSpecZVariants = 4;     // ... per z pass
 template <typename R> cudaError_t spec_axis(const AxisArgs &a, cudaStream_t s);
+// Two inputs, one output (the adjoint's passes), sizes with specialised
+// kernels only: inv 0, forward y: dst[0] = i m_y Y[src] + i m_z Y[src2];
+// inv 1: dst[0] = X^-1[-T(m2) (i m_x X[src] + X[src2])], T = table / interp.
+template <typename R> cudaError_t spec_axis_dual(const AxisArgs &a, cudaStream_t s);
 // Tile width (complex columns) of the size-specialised strided pass at n in
 // tile variant v (0 when n has no specialised kernels).
 template <typename R> int spec_axis_cols(int n, int v);
