@@ -214,9 +214,9 @@ gg_status gg_plan_variants(const gg_plan_t *plan, int32_t out[6]);
 gg_status gg_plan_set_variants(gg_plan_t *plan, const int32_t v[6]);
 
 /* Layout of the spectrum between the y forward and the y inverse passes of
- * a three-component run (pos and/or vel of all components, no psi output,
- * no Sec. 2.4 cut): 0 plain [x][y][k_z]; 1 chunk-major [k_z chunk][x][y]
- * [tile width], in which a tile of the x pass spans a few hundred kilobytes
+ * a three-component run (any output of every component, no Sec. 2.4 cut; a
+ * new plan takes the faster of the two by its size): 0 plain [x][y][k_z];
+ * 1 chunk-major [k_z chunk][x][y][tile width], in which a tile of the x pass spans a few hundred kilobytes
  * per chunk instead of one memory page per row. Results are bit-identical
  * (same arithmetic in the same order). The chunk-major layout needs the four
  * strided passes' variants to share a tile width; otherwise the plain one

@@ -359,6 +359,34 @@ void choose_tiles(gg_plan_t *plan) {
   plan->col_rows_box = (sizeof(R) == 8 || half % 2 == 0) && (size_t)b * cb >= 16 ? rows : 0;
 }
 
+// The tile variants and the layout a new plan starts with (gg_autotune and the
+// setters replace them; results do not depend on them). FP32 sizes with
+// variants, us per pass of a noise -> pos + vel run, variant 0 -> the one
+// taken, one realization each:
+// * z passes: warp barriers, with half the lines per CTA up to N = 256
+//   (N = 128: 12.4 + 35.5 -> 11.5 + 31.6; 256: 49.5 + 123.5 -> 46.0 + 119.7) and
+//   all of them above (384: 157.9 + 357 -> 147.6 + 356; 512: 336 + 784 -> 310 +
+//   775; 1536: 9849 + 21987 -> 9639 + 21844);
+// * x fused: the small tile where three of its CTAs fit an SM (512: 456 -> 420);
+// * y inverses: the small tile, two CTAs an SM, between 256 and 512 (384: 90 +
+//   150 -> 79 + 119); at 512 the two-output one alone, by variant 1 (272 ->
+//   261); elsewhere variant 0 is within 3% of the best.
+// * chunk-major spectra where a row of the x pass's tiles is 2 MB (a memory
+//   page) or more from the next: 768: 7953 -> 7917; 1024: 23050 -> 21640; 1536:
+//   69980 -> 66990 a run (512, rows of 1 MB: 2191 -> 2178, but its x pass's tile
+//   is narrower than the others').
+void default_shapes(gg_plan_t *plan) {
+  const int n = (int)plan->p.n;
+  if (plan->real_bytes != 4 || !gg::spec_has<float>(n)) return;
+  plan->chunked = (int64_t)n * (n / 2) * 8 >= ((int64_t)2 << 20);
+  if (!gg::spec_tuned<float>(n)) return;
+  plan->variant[0] = plan->variant[5] = n <= 256 ? 3 : 2;
+  plan->variant[2] = gg::spec_three_ctas<float>(n) ? 2 : 0;
+  const bool mid = n > 256 && n < 512;
+  plan->variant[3] = mid ? 2 : 0;
+  plan->variant[4] = mid ? 2 : (n == 512 ? 1 : 0);
+}
+
 void release(gg_plan_t *plan) {
   if (!plan) return;
   void *bufs[] = {plan->work,        plan->work2,         plan->work3,
@@ -584,23 +612,28 @@ int chunk_cols(gg_plan_t *plan) {
   return b;
 }
 
-// Positions and velocities of all three components with the spectrum
-// chunk-major between the y forward and the y inverse passes ([k_z chunk][x]
-// [y][cols]): a tile of the x pass, and the concurrent tiles around it, then
-// span a few hundred kilobytes of each chunk instead of one memory page per
-// row. Same arithmetic as the plain chain, in the same order; only the
-// buffers differ:
-//   y forward  work -> work3 (chunk-major)
-//   x fused    work3 -> A: work3 (in place), B: work2 (both chunk-major)
-//   y inverse  work3 -> work (plain); z inverse x from work
-//   y inverse  work2 -> work (i m_y), work3; z inverses y, z
+// All three components with the spectrum chunk-major between the y forward
+// and the y inverse passes ([k_z chunk][x][y][cols]): a tile of the x pass,
+// and the concurrent tiles around it, then span a few hundred kilobytes of
+// each chunk instead of one memory page per row. Same arithmetic as the plain
+// chain, in the same order; only the buffers differ (b2, b3: psi_y and psi_z
+// where they are wanted, else the plan's work2 and work3):
+//   y forward  work -> b3 (chunk-major)
+//   x fused    b3 -> A: b3 (in place), B: b2 (both chunk-major)
+//   y inverse  b3 -> work (plain); z inverse x from work
+//   y inverse  b2 -> work (i m_y), b3; z inverses y, z
 template <typename R>
 gg_status run_zeldovich_chunked(gg_plan_t *plan, uint64_t seed, const void *noise,
-                                void *const pos[3], void *const vel[3]) {
+                                void *const psi[3], void *const pos[3], void *const vel[3]) {
   const int b = chunk_cols<R>(plan);
-  gg_status st = forward_zy<R>(plan, seed, noise, plan->work3, b);
-  if (st != GG_OK) return st;
-  gg::AxisArgs x = axis_args<R>(plan, 0, plan->work3);
+  gg_status st;
+  void *b2 = psi && psi[1] ? psi[1] : nullptr, *b3 = psi && psi[2] ? psi[2] : nullptr;
+  if (!b2 && (st = ensure_grid(plan, &plan->work2)) != GG_OK) return st;
+  if (!b3 && (st = ensure_grid(plan, &plan->work3)) != GG_OK) return st;
+  if (!b2) b2 = plan->work2;
+  if (!b3) b3 = plan->work3;
+  if ((st = forward_zy<R>(plan, seed, noise, b3, b)) != GG_OK) return st;
+  gg::AxisArgs x = axis_args<R>(plan, 0, b3);
   x.cols = b;
   x.fwd = 1;
   x.inv = 1;
@@ -609,15 +642,15 @@ gg_status run_zeldovich_chunked(gg_plan_t *plan, uint64_t seed, const void *nois
   x.interp = plan->tab.interp_u;
   x.interp_cells = plan->tab.interp_cells;
   x.nout = 2;
-  x.dst[0] = plan->work3;
+  x.dst[0] = b3;
   x.mul[0] = gg::kMulIm;
-  x.dst[1] = plan->work2;
+  x.dst[1] = b2;
   x.mul[1] = gg::kMulNone;
   x.chunked_in = 1;
   x.chunked_out = 1;
   x.variant = plan->variant[2];
   if ((st = launch_axis_timed<R>(plan, x, kXFused, "x fused pass")) != GG_OK) return st;
-  gg::AxisArgs y = axis_args<R>(plan, 1, plan->work3);
+  gg::AxisArgs y = axis_args<R>(plan, 1, b3);
   y.cols = b;
   y.inv = 1;
   y.nout = 1;
@@ -627,23 +660,23 @@ gg_status run_zeldovich_chunked(gg_plan_t *plan, uint64_t seed, const void *nois
   y.variant = plan->variant[3];
   if ((st = launch_axis_timed<R>(plan, y, kYInvX, "y inverse pass (x branch)")) != GG_OK) return st;
   auto out = [&](void *const *a, int j) { return a ? a[j] : nullptr; };
-  if ((st = zinv_pass<R>(plan, 0, plan->work, nullptr, out(pos, 0), out(vel, 0), false)) != GG_OK)
+  if ((st = zinv_pass<R>(plan, 0, plan->work, out(psi, 0), out(pos, 0), out(vel, 0), false)) != GG_OK)
     return st;
-  gg::AxisArgs y2 = axis_args<R>(plan, 1, plan->work2);
+  gg::AxisArgs y2 = axis_args<R>(plan, 1, b2);
   y2.cols = b;
   y2.inv = 1;
   y2.nout = 2;
   y2.dst[0] = plan->work;
   y2.mul[0] = gg::kMulIm;
-  y2.dst[1] = plan->work3;
+  y2.dst[1] = b3;
   y2.mul[1] = gg::kMulNone;
   y2.chunked_in = 1;
   y2.variant = plan->variant[4];
   if ((st = launch_axis_timed<R>(plan, y2, kYInvYZ, "y inverse pass (y/z branches)")) != GG_OK)
     return st;
-  if ((st = zinv_pass<R>(plan, 1, plan->work, nullptr, out(pos, 1), out(vel, 1), false)) != GG_OK)
+  if ((st = zinv_pass<R>(plan, 1, plan->work, out(psi, 1), out(pos, 1), out(vel, 1), false)) != GG_OK)
     return st;
-  return zinv_pass<R>(plan, 2, plan->work3, nullptr, out(pos, 2), out(vel, 2), true);
+  return zinv_pass<R>(plan, 2, b3, out(psi, 2), out(pos, 2), out(vel, 2), true);
 }
 
 // Everything up to the inverse z passes. On return src[j] holds, for each
@@ -725,13 +758,8 @@ gg_status run_zeldovich(gg_plan_t *plan, uint64_t seed, const void *noise, void 
   for (int j = 0; j < 3; ++j)
     want[j] = (psi && psi[j]) || (pos && pos[j]) || (vel && vel[j]);
   if (!want[0] && !want[1] && !want[2]) return GG_OK;
-  const bool any_psi = psi && (psi[0] || psi[1] || psi[2]);
-  if (plan->chunked && !any_psi && want[0] && want[1] && want[2] && chunk_cols<R>(plan) > 0) {
-    gg_status st = GG_OK;
-    if ((st = ensure_grid(plan, &plan->work2)) != GG_OK) return st;
-    if ((st = ensure_grid(plan, &plan->work3)) != GG_OK) return st;
-    return run_zeldovich_chunked<R>(plan, seed, noise, pos, vel);
-  }
+  if (plan->chunked && want[0] && want[1] && want[2] && chunk_cols<R>(plan) > 0)
+    return run_zeldovich_chunked<R>(plan, seed, noise, psi, pos, vel);
   void *src[3];
   gg_status st = spectral_passes<R>(plan, seed, noise, want, psi, src);
   if (st != GG_OK) return st;
@@ -788,6 +816,7 @@ gg_status create(gg_plan_t *plan, const gg::cosmo::Model &m) {
   cudaError_t e = cudaMemset(plan->err, 0, 256);
   if (e != cudaSuccess) return cuda_fail(plan, e, "cudaMemset");
   choose_tiles<R>(plan);
+  default_shapes(plan);
   plan->info.workspace_bytes = (int64_t)workspace_bytes(&plan->p);
   return GG_OK;
 }
@@ -2006,6 +2035,9 @@ gg_status gg_batch_plan(gg_batch_t **batch, const gg_params *params, int count, 
   for (auto &g : b->groups) {
     const gg_params &p = params[g.members[0]];
     if ((st = gg_plan(&g.plan, &p, stream)) != GG_OK) break;
+    // several realizations a launch, groups side by side: variant 0 throughout
+    // (16 realizations of 128 .. 384: 5.58 ms, 5.64 with a lone run's choice)
+    for (int &v : g.plan->variant) v = 0;
     const size_t nb = g.members.size();
     const size_t bytes = (size_t)p.n * p.n * p.n * (p.prec == GG_F64 ? 8 : 4) * nb;
     for (void *&w : g.work)

@@ -9,6 +9,7 @@ namespace gg {
 using TableF32 = CtTable<float, 64, 128, 192, 256, 384, 512, 1536>;
 template <> bool spec_has<float>(int n) { return TableF32::has(n) || spec_more_has_f32(n); }
 template <> bool spec_tuned<float>(int n) { return TableF32::has(n); }
+template <> bool spec_three_ctas<float>(int n) { return TableF32::three(n); }
 template <> cudaError_t spec_axis<float>(const AxisArgs &a, cudaStream_t s) {
   return TableF32::has(a.n) ? TableF32::axis(a, s) : spec_more_axis_f32(a, s);
 }

@@ -1071,6 +1071,7 @@ constexpr int kZVariants = 4;
 // Run-time dispatch over the specialised sizes and their tile variants.
 template <typename R, int... NS> struct CtTable {
   static bool has(int n) { return ((n == NS) || ...); }
+  static bool three(int n) { return ((n == NS && ct::AxisPolicy<R, NS, 2>::THREE) || ...); }
   template <int N> static int cols_n(int v) {
     if constexpr (!ct::ct_tuned<R>(N)) return ct::AxisPolicy<R, N, 0>::B;
     else return v == 1 ? ct::AxisPolicy<R, N, 1>::B : (v == 2 ? ct::AxisPolicy<R, N, 2>::B : ct::AxisPolicy<R, N, 0>::B);

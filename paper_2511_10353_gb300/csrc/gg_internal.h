@@ -239,6 +239,7 @@ template <typename R> int max_block_threads_axis(int e);
 // the named workloads; spec_has tells whether N has them.
 template <typename R> bool spec_has(int n);
 template <typename R> bool spec_tuned(int n);  // has tile variants (gg_autotune)
+template <typename R> bool spec_three_ctas(int n);  // strided variant 2: three CTAs an SM
 // the F32 sizes with one tile shape (gg_ct_more_f32.cu, gg_ct_more_z_f32.cu)
 #define GG_MORE_F32 32, 48, 72, 96, 144, 216, 288, 432, 576, 648, 768, 864, 1024, 1152
 bool spec_more_has_f32(int n);
