@@ -13,6 +13,9 @@ template <> bool spec_three_ctas<float>(int n) { return TableF32::three(n); }
 template <> cudaError_t spec_axis<float>(const AxisArgs &a, cudaStream_t s) {
   return TableF32::has(a.n) ? TableF32::axis(a, s) : spec_more_axis_f32(a, s);
 }
+cudaError_t spec_axis_filter_f32(const AxisArgs &a, cudaStream_t s) {
+  return TableF32::has(a.n) ? TableF32::axis_filter(a, s) : spec_more_axis_filter_f32(a, s);
+}
 template <> int spec_axis_cols<float>(int n, int v) {
   return TableF32::has(n) ? TableF32::cols(n, v) : spec_more_cols_f32(n, v);
 }

@@ -29,7 +29,10 @@ __device__ __forceinline__ int ct_freq(int n, int N) { return n < (N >> 1) ? n :
 // a.interp say, kFiltNone never (the forward y pass), kFiltInterp always by the
 // interpolated FP32 table at a.interp (the fused x pass of the plain path).
 constexpr int kAxisFwd = 1, kAxisInv = 2, kAxisFwdInv = 3;
-constexpr int kFiltArgs = 0, kFiltNone = 1, kFiltInterp = 2;
+// kFiltAxis: by the complex factor a.table[n] of the pass axis alone (separable
+// filters on real fields: the packed pairs (2k, 2k+1) of a line are two real
+// columns, on which a Hermitian factor acts alike).
+constexpr int kFiltArgs = 0, kFiltNone = 1, kFiltInterp = 2, kFiltAxis = 3;
 // The body processes tiles t0, t0 + tstep, ... below tlimit (the kernel: its
 // CTA's share of all tiles; the persistent batched kernel: one tile). It
 // returns false when a copy wait gave up (the error word then holds
@@ -94,7 +97,7 @@ __device__ __forceinline__ bool axis_body(const CUtensorMap &map, const AxisArgs
   const int64_t ntiles = per_real * (a.nbatch > 0 ? a.nbatch : 1);
   const R *table = reinterpret_cast<const R *>(a.table);
   static_assert(FILT != kFiltInterp || sizeof(R) == 4, "interpolated filter: FP32");
-  const bool pre = FILT == kFiltArgs ? a.pre != 0 : FILT == kFiltInterp;
+  const bool pre = FILT == kFiltArgs ? a.pre != 0 : FILT == kFiltInterp || FILT == kFiltAxis;
   const bool interp = FILT == kFiltArgs ? sizeof(R) == 4 && a.pre && a.interp : FILT == kFiltInterp;
   // large radices: the N twiddles in shared memory (15-31 loads a butterfly),
   // after the tiles and the filter table
@@ -191,7 +194,7 @@ __device__ __forceinline__ bool axis_body(const CUtensorMap &map, const AxisArgs
       const int m = ct_freq(n, N);
       return (n == HALF || nyq_outer) ? -1 : m * m + m_outer * m_outer + kz * kz;
     };
-    if (pre && !interp) {
+    if (FILT != kFiltAxis && pre && !interp) {
 #pragma unroll
       for (int b = 0; b < NB; ++b)
 #pragma unroll
@@ -262,7 +265,14 @@ __device__ __forceinline__ bool axis_body(const CUtensorMap &map, const AxisArgs
 #pragma unroll
         for (int r = 0; r < RH; ++r) X[b * RH + r] = buf[(p + P * b + r * SPAN) * B + c];
     }
-    if (pre) {
+    if constexpr (FILT == kFiltAxis) {
+      const C *fac = reinterpret_cast<const C *>(a.table);
+#pragma unroll
+      for (int b = 0; b < NB; ++b)
+#pragma unroll
+        for (int r = 0; r < RH; ++r)
+          X[b * RH + r] = cmul(X[b * RH + r], ldg_c(fac + p + P * b + r * SPAN));
+    } else if (pre) {
 #pragma unroll
       for (int b = 0; b < NB; ++b)
 #pragma unroll
@@ -970,7 +980,111 @@ __global__ void __launch_bounds__(ct::ZPolicy<R, N, V>::THREADS,
   zfwd_body<R, N, V, NOISE>(a, blockIdx.x, gridDim.x, INT64_MAX);
 }
 
+// Separable spectral filter, z axis: real lines in, r2c, X_k times the complex
+// factor F_k (0 <= k < N/2; the z-Nyquist mode is dropped), c2r, real lines out
+// (in place allowed). One pass instead of the forward and the inverse one:
+// HBM-bound at 8 B/cell. The unpacking and packing of a conjugate pair meet in
+// registers: with X'_k = F_k X_k, S = X'_k + conj X'_{M-k}, D = X'_k - conj
+// X'_{M-k} and T = i D conj w_k, Z'_k = S + T and Z'_{M-k} = conj(S - T).
+template <typename R, int N>
+__global__ void __launch_bounds__(ct::ZPolicy<R, N, 0>::THREADS, ct::ZPolicy<R, N, 0>::MINB_NOISE)
+    k_zfilter(const ZFilterArgs a) {
+  using C = Cx<R>;
+  using Pol = ct::ZPolicy<R, N, 0>;
+  constexpr int M = Pol::M, E = Pol::E, P = Pol::P, L = Pol::L, LD = Pol::LD_FWD, PAD = Pol::PAD_FWD;
+  constexpr int KM = ct::skey<R>(M);
+  constexpr int S = ct::nstages(KM);
+  constexpr int RL = ct::radix_of(KM, S - 1, true), SPANL = M / RL, NBL = E / RL;
+  constexpr int DENSE_STRIDE = (int)(((Pol::DENSE * sizeof(C) + 127) / 128) * 128 / sizeof(C));
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  uint64_t *bar = reinterpret_cast<uint64_t *>(smem_raw);
+  C *dense = reinterpret_cast<C *>(smem_raw + 128);
+  C *work = dense + DENSE_STRIDE;
+  const int tid = threadIdx.x;
+  const int64_t ntiles = a.nlines / L;
+  const ct::Tw<C, false> tw_half{reinterpret_cast<const C *>(a.tw_half)};
+  const C *twf = reinterpret_cast<const C *>(a.tw_full), *fac = reinterpret_cast<const C *>(a.factor);
+  if (tid == 0) {
+    mbar_init(bar, 1);
+    fence_mbar_init();
+  }
+  __syncthreads();
+  auto issue = [&](int64_t t) {
+    mbar_arrive_expect_tx(bar, (uint32_t)(Pol::DENSE * sizeof(C)));
+    bulk_load(dense, reinterpret_cast<const C *>(a.src) + t * Pol::DENSE,
+              (uint32_t)(Pol::DENSE * sizeof(C)), bar);
+  };
+  int64_t t = blockIdx.x;
+  if (tid == 0 && t < ntiles) issue(t);
+  uint32_t phase = 0;
+  for (; t < ntiles; t += gridDim.x, phase ^= 1) {
+    int l = tid / P, p = tid - (tid / P) * P;
+    asm volatile("" : "+r"(l), "+r"(p));
+    __builtin_assume(l >= 0 && l < L && p >= 0 && p < P);
+    const bool ok = __syncthreads_and(mbar_wait(bar, phase, a.err));
+    if (!ok) return;  // nothing else in flight: the next copy is issued after this wait
+    const C *dl = dense + l * M;
+    auto ld_d = [&](int n) { return dl[n]; };
+    auto ld_w = [&](int n) { return work[zpad<LD, PAD>(l, n)]; };
+    auto st_w = [&](int n, C v) { work[zpad<LD, PAD>(l, n)] = v; };
+    ct::stage<R, M, E, 0, false, ct::kSyncNone>(p, tw_half, ld_d, st_w);
+    __syncthreads();
+    if (tid == 0 && t + gridDim.x < ntiles) {  // the dense tile has been read
+      fence_proxy_async_smem();
+      issue(t + gridDim.x);
+    }
+    ct::stages<R, M, E, false, 1, S, ct::kSyncCta>(p, tw_half, ld_w, st_w);
+    static_assert(P * (E / 2) == M / 2, "conjugate pairs");
+#pragma unroll
+    for (int i = 0; i < E / 2; ++i) {  // both members of a pair in one thread, in place
+      const int k = p + P * i;
+      const C zk = ld_w(k);
+      if (k == 0) {
+        const C zh = ld_w(M / 2);
+        const C x0 = {zk.x + zk.y, (R)0};
+        const C y0 = cmul(x0, ldg_c(fac)), yh = cmul(C{zh.x, -zh.y}, ldg_c(fac + M / 2));
+        st_w(0, C{y0.x, y0.x});
+        st_w(M / 2, C{(R)2 * yh.x, (R)-2 * yh.y});
+      } else {
+        const C zm = ld_w(M - k);
+        const C w = ldg_c(twf + k);
+        const C u = {(R)0.5 * w.y, (R)-0.5 * w.x};  // -(i/2) w, exact
+        const C sm = {zk.x + zm.x, zk.y - zm.y};
+        const C df = {zk.x - zm.x, zk.y + zm.y};
+        const C v = cmul(df, u);
+        const C xk = cmul(C{(R)0.5 * sm.x + v.x, (R)0.5 * sm.y + v.y}, ldg_c(fac + k));
+        const C xm = cmul(C{(R)0.5 * sm.x - v.x, v.y - (R)0.5 * sm.y}, ldg_c(fac + M - k));
+        const C s = {xk.x + xm.x, xk.y - xm.y}, d = {xk.x - xm.x, xk.y + xm.y};
+        const C q = mul_pi(cmulc(d, w));
+        st_w(k, C{s.x + q.x, s.y + q.y});
+        st_w(M - k, C{s.x - q.x, q.y - s.y});
+      }
+    }
+    __syncthreads();
+    ct::stages<R, M, E, true, 0, S - 1, ct::kSyncCta>(p, tw_half, ld_w, st_w);
+    C v[E];
+    ct::last_stage_regs<R, M, E, true>(p, tw_half, ld_w, v);
+    C *dst = reinterpret_cast<C *>(a.dst) + (t * L + l) * M;
+#pragma unroll
+    for (int b = 0; b < NBL; ++b)
+#pragma unroll
+      for (int r = 0; r < RL; ++r) dst[p + P * b + r * SPANL] = v[b * RL + r];
+    __syncthreads();  // the work tile's lines are rewritten next tile
+  }
+}
+
 // ------------------------------------------------------------ launchers
+template <typename R, int N> cudaError_t ct_launch_zfilter(const ZFilterArgs &a, cudaStream_t s) {
+  using Pol = ct::ZPolicy<R, N, 0>;
+  const size_t dense = (Pol::DENSE * 2 * sizeof(R) + 127) & ~(size_t)127;
+  const size_t smem = 128 + dense + (size_t)Pol::WORK_FWD * 2 * sizeof(R);
+  auto kern = k_zfilter<R, N>;
+  cudaError_t e = set_smem(kern, smem);
+  if (e != cudaSuccess) return e;
+  kern<<<persistent_blocks(kern, Pol::THREADS, smem, a.nlines / Pol::L), Pol::THREADS, smem, s>>>(a);
+  return cudaGetLastError();
+}
+
 template <typename R, int N, int V, int MODE, bool CUT = false, int FILT = kFiltArgs>
 cudaError_t ct_launch_axis(const AxisArgs &in, cudaStream_t s) {
   using Pol = ct::AxisPolicy<R, N, V>;
@@ -1116,6 +1230,21 @@ template <typename R, int... NS> struct CtTable {
   static cudaError_t dual(const AxisArgs &a, cudaStream_t s) {
     cudaError_t e = cudaErrorInvalidValue;
     ((a.n == NS ? (e = a.inv ? ct_launch_dual<R, NS, kDualX>(a, s) : ct_launch_dual<R, NS, kDualY>(a, s), 0) : 0), ...);
+    return e;
+  }
+  // one axis of a separable filter: strided (a.axis 0 or 1, factor in a.table), or z
+  template <int N> static cudaError_t axis_filter_n(const AxisArgs &a, cudaStream_t s) {
+    constexpr int V = ct::AxisPolicy<R, N, 2>::THREE ? 2 : 0;
+    return ct_launch_axis<R, N, V, kAxisFwdInv, false, kFiltAxis>(a, s);
+  }
+  static cudaError_t axis_filter(const AxisArgs &a, cudaStream_t s) {
+    cudaError_t e = cudaErrorInvalidValue;
+    ((a.n == NS ? (e = axis_filter_n<NS>(a, s), 0) : 0), ...);
+    return e;
+  }
+  static cudaError_t zfilter(const ZFilterArgs &a, cudaStream_t s) {
+    cudaError_t e = cudaErrorInvalidValue;
+    ((a.n == NS ? (e = ct_launch_zfilter<R, NS>(a, s), 0) : 0), ...);
     return e;
   }
   template <int N, int V> static cudaError_t zinv_v(const ZInvArgs &a, cudaStream_t s) {

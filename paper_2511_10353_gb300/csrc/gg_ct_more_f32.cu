@@ -12,6 +12,7 @@ namespace gg {
 using MoreF32 = CtTable<float, GG_MORE_F32>;
 bool spec_more_has_f32(int n) { return MoreF32::has(n); }
 int spec_more_cols_f32(int n, int v) { return MoreF32::cols(n, v); }
+cudaError_t spec_more_axis_filter_f32(const AxisArgs &a, cudaStream_t s) { return MoreF32::axis_filter(a, s); }
 cudaError_t spec_more_axis_f32(const AxisArgs &a, cudaStream_t s) { return MoreF32::axis(a, s); }
 
 }  // namespace gg

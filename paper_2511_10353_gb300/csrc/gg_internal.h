@@ -120,6 +120,19 @@ struct ZFwdArgs {
   int *err;               // device error word (caller noise: a copy wait gave up)
 };
 
+// One axis of a separable spectral filter on real lines along z (F32 sizes with
+// specialised kernels): r2c, X_k times factor[k], c2r; src may equal dst.
+struct ZFilterArgs {
+  const void *src;
+  void *dst;
+  const void *factor;     // N/2 complex
+  int64_t nlines;         // N^2
+  int n;
+  const void *tw_half;
+  const void *tw_full;
+  int *err;
+};
+
 // Inverse z pass (c2r) with the Zel'dovich epilogue (Eq. 3) or a plain real
 // output (density).
 struct ZInvArgs {
@@ -246,6 +259,8 @@ bool spec_more_has_f32(int n);
 int spec_more_cols_f32(int n, int v);
 cudaError_t spec_more_axis_f32(const AxisArgs &a, cudaStream_t s);
 cudaError_t spec_more_dual_f32(const AxisArgs &a, cudaStream_t s);
+cudaError_t spec_more_axis_filter_f32(const AxisArgs &a, cudaStream_t s);
+cudaError_t spec_more_zfilter_f32(const ZFilterArgs &a, cudaStream_t s);
 cudaError_t spec_more_zinv_f32(const ZInvArgs &a, cudaStream_t s);
 cudaError_t spec_more_zfwd_f32(const ZFwdArgs &a, cudaStream_t s);
 constexpr int kSpecAxisVariants = 3;  // tile variants the autotuner times per strided pass
@@ -255,6 +270,11 @@ template <typename R> cudaError_t spec_axis(const AxisArgs &a, cudaStream_t s);
 // kernels only: inv 0, forward y: dst[0] = i m_y Y[src] + i m_z Y[src2];
 // inv 1: dst[0] = X^-1[-T(m2) (i m_x X[src] + X[src2])], T = table / interp.
 template <typename R> cudaError_t spec_axis_dual(const AxisArgs &a, cudaStream_t s);
+// One axis of a separable filter on a real field, F32 sizes with specialised
+// kernels: the strided pass (axis 0 or 1; forward, X[n] times the complex
+// table[n], inverse, to dst[0]) and the z pass.
+cudaError_t spec_axis_filter_f32(const AxisArgs &a, cudaStream_t s);
+cudaError_t spec_zfilter_f32(const ZFilterArgs &a, cudaStream_t s);
 // Tile width (complex columns) of the size-specialised strided pass at n in
 // tile variant v (0 when n has no specialised kernels).
 template <typename R> int spec_axis_cols(int n, int v);
