@@ -26,8 +26,8 @@ SOURCES = [
     "gg_ct_z_f32.cu",
     "gg_ct_more_f32.cu",
     "gg_ct_more_z_f32.cu",
-    "gg_ct_f64.cu",
-    "gg_ct_z_f64.cu",
+    "gg_fx_axis.cu",
+    "gg_fx_z.cu",
     "gg_axis_f32.cu",
     "gg_axis_f64.cu",
     "gg_kernels_f32.cu",

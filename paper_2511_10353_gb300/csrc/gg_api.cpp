@@ -247,6 +247,12 @@ std::vector<R> twiddles(int len) {
   return t;
 }
 
+std::vector<int32_t> fixed_table(int len) {
+  std::vector<int32_t> t(4 * (size_t)len);
+  gg::fixed_twiddles(len, t.data());
+  return t;
+}
+
 template <typename R>
 gg_status upload(gg_plan_t *plan, void **dst, const std::vector<R> &v) {
   cudaError_t e = cudaMalloc(dst, v.size() * sizeof(R));
@@ -305,8 +311,13 @@ template <typename R>
 gg_status build_tables(gg_plan_t *plan, const gg::cosmo::Model &m) {
   const int64_t n = plan->p.n;
   gg_status st;
-  if ((st = upload(plan, &plan->tab.tw_n, twiddles<R>((int)n))) != GG_OK) return st;
-  if ((st = upload(plan, &plan->tab.tw_half, twiddles<R>((int)(n / 2)))) != GG_OK) return st;
+  if (sizeof(R) == 8 && gg::spec_has<double>((int)n)) {  // fixed-point transforms
+    if ((st = upload(plan, &plan->tab.tw_n, fixed_table((int)n))) != GG_OK) return st;
+    if ((st = upload(plan, &plan->tab.tw_half, fixed_table((int)(n / 2)))) != GG_OK) return st;
+  } else {
+    if ((st = upload(plan, &plan->tab.tw_n, twiddles<R>((int)n))) != GG_OK) return st;
+    if ((st = upload(plan, &plan->tab.tw_half, twiddles<R>((int)(n / 2)))) != GG_OK) return st;
+  }
   const size_t cnt = table_entries(n);
   std::vector<double> s(cnt);
   filter_values(&plan->p, m, plan->info.growth, s.data(), (int64_t)cnt);
@@ -1061,13 +1072,15 @@ gg_status run_adjoint3(gg_plan_t *plan, const void *const g_psi[3], void *g_nois
   return zinv_pass<R>(plan, 0, plan->work, g_noise, nullptr, nullptr, false);
 }
 
-// Some gradients only, or a size without specialised kernels: the forward
-// chain once per component, accumulated with weight -1.
+// Some gradients only, FP64, or a size without specialised kernels: the
+// forward chain once per component, accumulated with weight -1.
 template <typename R>
 gg_status run_adjoint(gg_plan_t *plan, const void *const g_psi[3], void *g_noise) {
-  if (g_psi && g_psi[0] && g_psi[1] && g_psi[2] && gg::spec_has<R>((int)plan->p.n)) {
-    const gg_status st = ensure_grid(plan, &plan->work2);
-    return st != GG_OK ? st : run_adjoint3<R>(plan, g_psi, g_noise);
+  if constexpr (sizeof(R) == 4) {
+    if (g_psi && g_psi[0] && g_psi[1] && g_psi[2] && gg::spec_has<R>((int)plan->p.n)) {
+      const gg_status st = ensure_grid(plan, &plan->work2);
+      return st != GG_OK ? st : run_adjoint3<R>(plan, g_psi, g_noise);
+    }
   }
   cudaError_t e = cudaMemsetAsync(g_noise, 0, (size_t)plan->cells * sizeof(R), plan->stream);
   if (e != cudaSuccess) return cuda_fail(plan, e, "cudaMemsetAsync");
@@ -1615,6 +1628,21 @@ bool info_and_filter(const gg_params *p, gg_info *info, double *s, int64_t count
   info->workspace_bytes = (int64_t)workspace_bytes(p);
   filter_values(p, m, info->growth, s, count);
   return true;
+}
+
+void fixed_twiddles(int len, int32_t *out) {
+  const long double pi = 3.14159265358979323846264338327950288L;
+  for (int t = 0; t < len; ++t) {
+    const long double ang = -2.0L * pi * (long double)t / (long double)len;
+    const long double v[2] = {std::cos(ang), std::sin(ang)};
+    for (int i = 0; i < 2; ++i) {
+      int64_t w = (int64_t)std::llroundl(v[i] * 4611686018427387904.0L);
+      if ((uint32_t)w == 0x80000000u) ++w;  // so that both halves can be negated
+      const int32_t lo = (int32_t)(uint32_t)w;
+      out[4 * t + 2 * i] = (int32_t)((w - lo) / 4294967296ll);
+      out[4 * t + 2 * i + 1] = lo;
+    }
+  }
 }
 
 bool make_stages(int len, FftStages *st) {

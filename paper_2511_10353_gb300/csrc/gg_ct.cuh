@@ -11,7 +11,7 @@
 
 #include <cuda.h>
 
-#include "gg_device.cuh"
+#include "gg_fx.cuh"
 
 namespace gg {
 namespace ct {
@@ -24,9 +24,11 @@ namespace ct {
 // shared-memory round trip and one twiddle stage instead of two or three of
 // each. Other lengths, and every FP64 codelet (whose bound is the FP64
 // pipe, not the stage count), use radix 8 first, then 4 or 2, then the 3s.
-constexpr int kBig = 1 << 20;
+// The fixed-point codelets of the FP64 sizes (kFx, R = long long) keep a thread
+// at 8 or 12 elements (four registers each) where the length allows it.
+constexpr int kBig = 1 << 20, kFx = 1 << 21;
 template <typename R> __host__ __device__ constexpr int skey(int n) {
-  return sizeof(R) == 4 ? (n | kBig) : n;
+  return sizeof(R) == 4 ? (n | kBig) : (std::is_same<R, long long>::value ? (n | kFx) : n);
 }
 __host__ __device__ constexpr int key_n(int key) { return key & (kBig - 1); }
 
@@ -68,13 +70,31 @@ __host__ __device__ constexpr int big_radix(int n, int s) {
     default: return 0;
   }
 }
-__host__ __device__ constexpr bool is_big(int key) {
-  return (key & kBig) != 0 && big_radix(key_n(key), 0) != 0;
+__host__ __device__ constexpr int fx_radix(int n, int s) {
+  switch (n) {
+    case 24: return s == 0 ? 4 : (s == 1 ? 6 : 0);
+    case 36: return s < 2 ? 6 : 0;
+    case 48: return s == 0 ? 4 : (s == 1 ? 12 : 0);
+    case 72: return s == 0 ? 6 : (s == 1 ? 12 : 0);
+    case 96: return s < 2 ? 4 : (s == 2 ? 6 : 0);
+    case 108: return s < 2 ? 6 : (s == 2 ? 3 : 0);
+    case 144: return s < 2 ? 12 : 0;
+    case 192: return s < 2 ? 4 : (s == 2 ? 12 : 0);
+    case 216: return s < 3 ? 6 : 0;
+    case 288: return s == 0 ? 4 : (s == 1 ? 6 : (s == 2 ? 12 : 0));
+    case 384: return s < 3 ? 4 : (s == 3 ? 6 : 0);
+    case 768: return s < 3 ? 4 : (s == 3 ? 12 : 0);
+    default: return 0;
+  }
 }
+__host__ __device__ constexpr int own_radix(int key, int s) {
+  return (key & kBig) ? big_radix(key_n(key), s) : ((key & kFx) ? fx_radix(key_n(key), s) : 0);
+}
+__host__ __device__ constexpr bool is_big(int key) { return own_radix(key, 0) != 0; }
 __host__ __device__ constexpr int nstages(int key) {
   if (is_big(key)) {
     int c = 0;
-    while (big_radix(key_n(key), c)) ++c;
+    while (own_radix(key, c)) ++c;
     return c;
   }
   const Fac f = factor(key_n(key));
@@ -82,7 +102,7 @@ __host__ __device__ constexpr int nstages(int key) {
 }
 // forward schedule: radix 8 first, then 4 or 2, then the 3s (or the large radices)
 __host__ __device__ constexpr int radix_fwd(int key, int s) {
-  if (is_big(key)) return big_radix(key_n(key), s);
+  if (is_big(key)) return own_radix(key, s);
   const Fac f = factor(key_n(key));
   const int n8 = f.a / 3;
   if (s < n8) return 8;
@@ -171,6 +191,22 @@ template <int RT, int EXP, bool INV, typename T> __device__ __forceinline__ T tw
     return mul_wi<INV>(a);  // -i forward
   } else if constexpr (4 * e == 3 * RT) {
     return mul_wi<!INV>(a);  // +i forward
+  } else if constexpr (std::is_same<T, Fx>::value) {
+    if constexpr ((8 * e) % RT == 0) {  // (+-1 +- i) / sqrt 2
+      constexpr int h = fx::high_half(fx::kSqrtHalf), l = fx::low_half(fx::kSqrtHalf);
+      constexpr int o = 8 * e / RT;  // 1, 3, 5, 7
+      constexpr bool cp = o == 1 || o == 7, sp = (o == 5 || o == 7) != INV;  // signs of re and im
+      const long long s = fx::mul_real(a.x + a.y, h, l), d = fx::mul_real(a.x - a.y, h, l);
+      // (a.x c - a.y s, a.x s + a.y c), |c| = |s| = h
+      if constexpr (cp && sp) return T{d, s};
+      else if constexpr (cp && !sp) return T{s, -d};
+      else if constexpr (!cp && sp) return T{-s, d};
+      else return T{-d, -s};
+    } else {
+      constexpr long long c = fx::units(cos_turn(e, RT));
+      constexpr long long sn = fx::units(INV ? sin_turn(e, RT) : -sin_turn(e, RT));
+      return fx::mul(a, fx::high_half(c), fx::low_half(c), fx::high_half(sn), fx::low_half(sn));
+    }
   } else if constexpr ((8 * e) % RT == 0) {  // (+-1 +- i) / sqrt 2
     constexpr R h = (R)0.70710678118654752440;
     constexpr int o = 8 * e / RT;  // 1, 3, 5, 7
@@ -274,7 +310,7 @@ __device__ __forceinline__ void stage_twiddles(Cx<R> *v, int k, Cx<R> w1, const 
   } else {
 #pragma unroll
     for (int r = 1; r < RAD; ++r) {
-      const Cx<R> w = tw[k * TSTEP * r];
+      const auto w = tw[k * TSTEP * r];
       v[r] = INV ? cmulc(v[r], w) : cmul(v[r], w);
     }
   }
@@ -414,7 +450,7 @@ __device__ __forceinline__ void stage_twiddle(Cx<R> *v, const TwT &tw, int kt) {
   } else {
 #pragma unroll
     for (int r = 1; r < RAD; ++r) {
-      const Cx<R> w = tw[kt * r];
+      const auto w = tw[kt * r];
       v[r] = INV ? cmulc(v[r], w) : cmul(v[r], w);
     }
   }

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "gg_gauss64.cuh"
 #include "gg_internal.h"
 
 namespace gg {
@@ -127,10 +128,9 @@ __device__ __forceinline__ void gauss2(uint32_t ra, uint32_t rb, float &c, float
   s = rho * sn;
 }
 __device__ __forceinline__ void gauss2(uint32_t ra, uint32_t rb, double &c, double &s) {
-  const double ua = ((double)ra + 1.0) * 0x1p-32;
-  const double rho = sqrt(-2.0 * log(ua));
+  const double rho = gauss64::root(gauss64::neg2_ln(ra));
   double sn, cs;
-  sincospi(2.0 * ((double)rb * 0x1p-32), &sn, &cs);
+  gauss64::sincos_turn(rb, sn, cs);
   c = rho * cs;
   s = rho * sn;
 }
@@ -160,6 +160,9 @@ __device__ __forceinline__ double fma_rn(double a, double b, double c) { return 
 // Periodic wrap of a coordinate into [0, L) (Eq. 3 positions).
 template <typename R>
 __device__ __forceinline__ R wrap_box(R x, R box) {
+  if constexpr (sizeof(R) == 8) {  // 0 <= x < box by the bits: no FP64 comparisons
+    if ((unsigned long long)__double_as_longlong(x) < (unsigned long long)__double_as_longlong(box)) return x;
+  }
   if (x < (R)0) x += box;
   else if (x >= box) x -= box;
   if (!(x >= (R)0 && x < box)) {

@@ -255,6 +255,12 @@ template <typename R> bool spec_tuned(int n);  // has tile variants (gg_autotune
 template <typename R> bool spec_three_ctas(int n);  // strided variant 2: three CTAs an SM
 // the F32 sizes with one tile shape (gg_ct_more_f32.cu, gg_ct_more_z_f32.cu)
 #define GG_MORE_F32 32, 48, 72, 96, 144, 216, 288, 432, 576, 648, 768, 864, 1024, 1152
+// the F64 sizes with specialised kernels (gg_fx_axis.cu, gg_fx_z.cu); their
+// twiddle tables are fixed_twiddles'
+#define GG_FX_SIZES 32, 48, 64, 72, 96, 128, 144, 192, 216, 256, 288, 384, 512, 768, 1024, 1536
+// exp(-2 pi i t / len), t < len, as four 32-bit integers each: round(re 2^62) =
+// out[4t] 2^32 + out[4t + 1], round(im 2^62) = out[4t + 2] 2^32 + out[4t + 3].
+void fixed_twiddles(int len, int32_t *out);
 bool spec_more_has_f32(int n);
 int spec_more_cols_f32(int n, int v);
 cudaError_t spec_more_axis_f32(const AxisArgs &a, cudaStream_t s);
@@ -266,7 +272,7 @@ cudaError_t spec_more_zfwd_f32(const ZFwdArgs &a, cudaStream_t s);
 constexpr int kSpecAxisVariants = 3;  // tile variants the autotuner times per strided pass
 constexpr int kSpecZVariants = 4;     // ... per z pass
 template <typename R> cudaError_t spec_axis(const AxisArgs &a, cudaStream_t s);
-// Two inputs, one output (the adjoint's passes), sizes with specialised
+// Two inputs, one output (the adjoint's passes), FP32 sizes with specialised
 // kernels only: inv 0, forward y: dst[0] = i m_y Y[src] + i m_z Y[src2];
 // inv 1: dst[0] = X^-1[-T(m2) (i m_x X[src] + X[src2])], T = table / interp.
 template <typename R> cudaError_t spec_axis_dual(const AxisArgs &a, cudaStream_t s);

@@ -96,11 +96,17 @@ gg_status run(const gg_params *p, const gg_info &info, const double *sd, uint64_
   const int n = (int)p->n, half = n / 2;
   // tables in FP64 on the host, rounded once, copied into the scratch arrays
   R tw_n[2 * kMaxN], tw_half[2 * kMaxHalf], tab[kMaxTable];
-  for (int i = 0; i < n; ++i) {
+  const bool spec = gg::spec_has<R>(n);
+  if (sizeof(R) == 8 && spec) {  // fixed-point transforms
+    static_assert(sizeof(double) == 2 * sizeof(int32_t), "four 32-bit integers a twiddle");
+    gg::fixed_twiddles(n, reinterpret_cast<int32_t *>(tw_n));
+    gg::fixed_twiddles(half, reinterpret_cast<int32_t *>(tw_half));
+  }
+  for (int i = 0; i < n && !(sizeof(R) == 8 && spec); ++i) {
     tw_n[2 * i] = (R)std::cos(-2.0 * kPi * i / n);
     tw_n[2 * i + 1] = (R)std::sin(-2.0 * kPi * i / n);
   }
-  for (int i = 0; i < half; ++i) {
+  for (int i = 0; i < half && !(sizeof(R) == 8 && spec); ++i) {
     tw_half[2 * i] = (R)std::cos(-2.0 * kPi * i / half);
     tw_half[2 * i + 1] = (R)std::sin(-2.0 * kPi * i / half);
   }
@@ -118,7 +124,6 @@ gg_status run(const gg_params *p, const gg_info &info, const double *sd, uint64_
   if (!gg::make_stages(n, &st_n) || !gg::make_stages(half, &st_half))
     return fail(GG_EINVAL, "gg_gaussian_field_static: no FFT schedule");
   const gg::FftStages st_inv = gg::reversed_stages(st_n);
-  const bool spec = gg::spec_has<R>(n);
   // z forward: noise (generated or read) -> half spectrum in the scratch grid
   gg::ZFwdArgs z{};
   z.noise = noise;
