@@ -39,12 +39,19 @@ __device__ __forceinline__ long long mul_real(long long a, int h, int l) {
   const int al = lo_of(a), ah = hi_of(a);
   return join((long long)ah * h, wide(al, h, wide(ah, l, kRound)));
 }
-// An integer rounded to FP64: its halves exactly in the mantissas of 2^84 and
-// 2^52 and two additions.
-__device__ __forceinline__ double rounded_double(long long f) {
-  const double a = __hiloint2double(0x45300000, (int)((uint32_t)(f >> 32) ^ 0x80000000u));
-  const double b = __hiloint2double(0x43300000, (int)(uint32_t)f);
-  return (a - (0x1p84 + 0x1p63 + 0x1p52)) + b;
+// An integer, times 2^-s, rounded to FP64 without the FP64 pipe: normalised,
+// rounded to nearest even and put together by integers (26 instructions; two exact
+// halves and two FP64 additions, 32 cycles of that pipe, took 13.9 instead of
+// 12.3 ms in the 512^3 FP64 run). |s| <= 960.
+__device__ __forceinline__ double scaled_double(long long f, int s) {
+  const long long sign = f >> 63;
+  const unsigned long long u = (unsigned long long)((f ^ sign) - sign);
+  const int z = __clzll((long long)u);
+  const unsigned long long n = u << (z & 63);  // bit 63 set
+  const uint32_t rest = ((uint32_t)n & 0x7ffu) + (((uint32_t)n >> 11) & 1u);  // ties to even
+  const unsigned long long m = (n >> 11) + (rest > 0x400u ? 1ull : 0ull);   // a carry goes on into the exponent
+  const uint32_t hi = (uint32_t)(m >> 32) + ((uint32_t)(1085 - z - s) << 20);
+  return __hiloint2double(u ? (int)(hi | ((uint32_t)(sign >> 32) & 0x80000000u)) : 0, (int)(uint32_t)m);
 }
 // halves of a constant of modulus below one in 2^62 units
 __host__ __device__ constexpr long long units(double c) {

@@ -5,8 +5,9 @@
 // instructions a point, 14 SM cycles, however it is scheduled, and the FP64
 // kernels ran at 84% of that bound. The same transform on 64-bit integers takes
 // about 120 integer instructions a point, two to three cycles. 512^3 noise ->
-// pos + vel 59.1 -> 13.9 ms (z forward 12.9 -> 2.95, y 3.38 -> 0.96, x 11.1 -> 3.35,
-// y inverses 11.0 -> 2.84, z inverses 20.7 -> 3.74).
+// pos + vel 59.1 -> 12.3 ms (z forward 12.9 -> 2.32, y 3.38 -> 0.86, x 11.1 -> 2.95,
+// y inverses 11.0 -> 2.54, z inverses 20.7 -> 3.61), bound by the latency of the
+// integer chains at 16 to 20 warps an SM.
 //
 // Each transform of N points (a column of a tile, a line) gets one power of two
 // as its scale, from the sum of |re| + |im| of its inputs (col_scale): the
@@ -139,14 +140,11 @@ __device__ __forceinline__ long long to_fixed(double v, const Scale &sc, const W
   return ((int)hi < 0) != w.neg ? -g : g;
 }
 
-// An integer in units of 2^-s rounded to FP64 (by two FP64 additions: that pipe
-// is otherwise idle); the power of two goes into the exponent.
+// An integer in units of 2^-s rounded to FP64.
 static __device__ __noinline__ double slow_scale(double v, int s) { return scalbn(v, -s); }
 __device__ __forceinline__ double to_double(long long f, const Scale &sc) {
-  const double v = rounded_double(f);
-  if (sc.s > 960 || sc.s < -960) return slow_scale(v, sc.s);
-  const int hw = __double2hiint(v);
-  return __hiloint2double(hw == 0 ? 0 : hw - (sc.s << 20), __double2loint(v));
+  if (sc.s > 960 || sc.s < -960) return slow_scale((double)f, sc.s);
+  return scaled_double(f, sc.s);
 }
 __device__ __forceinline__ double2 to_double2(const Fx &f, const Scale &sc) {
   double2 d = {to_double(f.x, sc), to_double(f.y, sc)};

@@ -1,8 +1,8 @@
 // FP64 Box-Muller on one word pair, for a GPU with two FP64 lanes an SM: the
 // arguments are 32-bit integers, so the logarithm, the sine and the cosine are
 // computed in 64-bit integers, and FP64 does the square root and the products
-// (14 instructions a pair instead of the 110 of log, sqrt and sincospi: the
-// 512^3 z forward pass 12.9 -> 2.95 ms together with its fixed-point transform).
+// (8 instructions a pair instead of the 110 of log, sqrt and sincospi: the
+// 512^3 z forward pass 12.9 -> 2.32 ms together with its fixed-point transform).
 //
 // * ln u, u = (r + 1) 2^-32 = y 2^(-1-z), y in [1, 2) from the 32 bits: the top
 //   seven fraction bits select c ~ 1/y (11 bits), t = y c - 1 is exact, ln u =
@@ -108,13 +108,6 @@ __host__ __device__ constexpr Tables make_tables() {
 }
 static __device__ const Tables kTables = make_tables();
 
-// integer in units of 2^-s to FP64 (rounded once)
-__device__ __forceinline__ double int_to_double(long long f, int s) {
-  const double v = fx::rounded_double(f);
-  const int hw = __double2hiint(v);
-  return __hiloint2double(hw == 0 ? 0 : hw - (s << 20), __double2loint(v));
-}
-
 __device__ __forceinline__ double neg2_ln_near1(uint32_t r) {  // u > 1 - 2^-8
   const double t = -((double)(~r) * 0x1p-32);                  // u - 1, exact
   double q = fma(t, 1.0 / 7.0, -1.0 / 6.0);
@@ -146,8 +139,8 @@ __device__ __forceinline__ double neg2_ln(uint32_t r) {  // -2 ln((r + 1) 2^-32)
   const long long l1 = (long long)((unsigned long long)t42 << 20) - (__mul64hi(t2, q) >> 12);  // ln(1 + t) 2^62
   const int n = z + (j < kRoot2 ? 1 : 0);
   // -2 ln u = 2 n ln 2 - 2 L - 2 ln(1 + t); 2 ln(1 + t) in units of 2^-61 is l1
-  if (n == 0) return int_to_double(w - l1, 61);
-  return int_to_double((long long)n * 199786072581291495ll + ((w - l1) >> 4), 57);
+  if (n == 0) return fx::scaled_double(w - l1, 61);
+  return fx::scaled_double((long long)n * 199786072581291495ll + ((w - l1) >> 4), 57);
 }
 __device__ __forceinline__ double root(double a) {  // sqrt(a), 0 or 2^-31 < a < 64
   const int hi = __double2hiint(a);
@@ -183,8 +176,8 @@ __device__ __forceinline__ void sincos_turn(uint32_t rb, double &s, double &c) {
   const long long cm = (x2 >> 1) - ((long long)__umulhi(x4, 178956971u) << 12);
   const Fx a = fx::mul(Fx{(1ll << 62) - (cm >> 14), sn >> 8}, e.x, e.y, e.z, e.w);
   const long long p = (q & 1) ? a.x : a.y, w = (q & 1) ? a.y : a.x;  // sin, cos by quarter turns
-  s = int_to_double((q & 2) ? -p : p, 62);
-  c = int_to_double(((q + 1) & 2) ? -w : w, 62);
+  s = fx::scaled_double((q & 2) ? -p : p, 62);
+  c = fx::scaled_double(((q + 1) & 2) ? -w : w, 62);
 }
 
 }  // namespace gauss64
