@@ -642,6 +642,15 @@ template <int LD, int PAD> __device__ __forceinline__ int zpad(int l, int n) {
   else return l * LD + n + (int)((unsigned)n / PAD);
 }
 
+// The merge's coarse lines in shared memory: most lines a tile of L z-lines needs
+// (they share x and follow each other in y), for interpolation between them;
+// 0 where the tile's lines do not share x. The lines are interpolated in x while
+// they are staged, so that a pair of cells reads 6 shared values instead of 12
+// through L1 (512^3 with a 256^3 coarse grid 578 -> 500 us, with an instantiation for pos + vel).
+template <int N, int L> __host__ __device__ constexpr int merge_rows(int nl) {
+  return N % L == 0 ? (int)(((int64_t)(L - 1) * nl + N - 1) / N) + 2 : 0;
+}
+
 // Inverse z pass (c2r) + Eq. 3 epilogue, persistent: one thread bulk-copies
 // a block of L contiguous half-spectrum lines into a dense shared buffer. The
 // c2r pre-processing moves it into the padded work tile (where the first two
@@ -685,6 +694,16 @@ __device__ __forceinline__ bool zinv_body(const ZInvArgs &a, int64_t t0, int64_t
   const int64_t ntiles = a.nlines / L;
   const ct::Tw<C, false> tw_half{reinterpret_cast<const C *>(a.tw_half)};
   const C *twf = reinterpret_cast<const C *>(a.tw_full);
+  // EXT: the coarse grid's lines around a tile (see merge_rows) and the z taps
+  // of every pair of cells
+  MergeTap<R> *taps = reinterpret_cast<MergeTap<R> *>(work + (Pol::WORK_INV + 1) / 2 * 2);
+  R *coarse = reinterpret_cast<R *>(taps + M);
+  const int nl2 = EXT ? a.n_low + 2 : 0;  // a staged line, its first two values repeated
+  if constexpr (EXT) {
+    if (a.large_rows) {
+      for (int n = tid; n < M; n += Pol::THREADS) taps[n] = merge_tap<R>(a.n_low, N, n);
+    }
+  }
   if (tid == 0) {
     mbar_init(bar, 1);
     fence_mbar_init();
@@ -705,6 +724,39 @@ __device__ __forceinline__ bool zinv_body(const ZInvArgs &a, int64_t t0, int64_t
     asm volatile("" : "+r"(l), "+r"(p));
     const bool ok = __syncthreads_and(mbar_wait(bar, (uint32_t)(it & 1), a.err));
     if (!ok) return false;  // nothing else in flight: the next copy is issued after this wait
+    int row0 = 0;  // EXT: coarse y of the first staged line
+    if constexpr (EXT) {
+      if (a.large_rows) {  // the tile's lines share x and follow each other in y
+        const uint32_t first = (uint32_t)(t * L) % (uint32_t)(a.lines_per_real > 0 ? a.lines_per_real : a.nlines);
+        const int x = (int)(first / (uint32_t)N), y = (int)(first - (uint32_t)x * (uint32_t)N);
+        const CicAxis<R> cx = cic_axis<R>(x, a.n_low, N);
+        row0 = cic_axis<R>(y, a.n_low, N).i0;
+        const R *g = reinterpret_cast<const R *>(a.large);
+        constexpr int BATCH = 6;  // rows whose loads are in flight together
+        for (int z = tid; z < a.n_low; z += Pol::THREADS)
+          for (int j0 = 0; j0 < a.large_rows; j0 += BATCH) {
+            R v0[BATCH], v1[BATCH];
+#pragma unroll
+            for (int j = 0; j < BATCH; ++j) {
+              int yy = row0 + j0 + j;
+              if (yy >= a.n_low) yy -= a.n_low;
+              if (yy >= a.n_low) yy -= a.n_low;
+              const bool on = j0 + j < a.large_rows;
+              v0[j] = on ? __ldg(g + ((int64_t)cx.i0 * a.n_low + yy) * a.n_low + z) : (R)0;
+              v1[j] = on ? __ldg(g + ((int64_t)cx.i1 * a.n_low + yy) * a.n_low + z) : (R)0;
+            }
+#pragma unroll
+            for (int j = 0; j < BATCH; ++j) {
+              if (j0 + j >= a.large_rows) break;
+              R *row = coarse + (j0 + j) * nl2;
+              const R v = ((R)1 - cx.t) * v0[j] + cx.t * v1[j];
+              row[z] = v;
+              if (z < 2) row[a.n_low + z] = v;
+              if (a.n_low == 1) row[2] = v;
+            }
+          }
+      }
+    }
     const C *dl = dense + l * M;
     const R pf = (R)p;  // (R)(p + c) == pf + (R)c exactly: small integers
     auto ld_w = [&](int n) { return work[zpad<LD, PAD>(l, n)]; };
@@ -791,24 +843,43 @@ __device__ __forceinline__ bool zinv_body(const ZInvArgs &a, int64_t t0, int64_t
         q1 = mul_rn(q2p + (R)(2 * (n - p) + 1) + qo, cell);
       }
     };
-    if constexpr (POSVEL) {
-      each([&](int n, C z) {
-        R q0, q1;
-        lattice(n, q0, q1);
-        pos[n] = C{wrap_box<R>(q0 + z.x, box), wrap_box<R>(q1 + z.y, box)};
-        vel[n] = C{vfac * z.x, vfac * z.y};
-      });
-    } else if constexpr (ONLY_PSI) {
-      each([&](int n, C z) { psi[n] = z; });
-    } else {
-      if constexpr (EXT) {  // Sec. 2.4: the interpolated coarse large scales
-        if (large) each([&](int n, C &z) {
+    if constexpr (EXT) {  // Sec. 2.4: the interpolated coarse large scales
+      if (a.large_rows) {  // from the staged lines (interpolated in x): y, then z
+        int j = cy.i0 - row0;
+        if (j < 0) j += a.n_low;
+        const R *r0 = coarse + j * nl2, *r1 = r0 + nl2;
+        const R w0 = (R)1 - cy.t, w1 = cy.t;
+        each([&](int n, C &z) {
+          const MergeTap<R> tap = taps[n];
+          const R c0 = w0 * r0[tap.z] + w1 * r1[tap.z];
+          const R c1 = w0 * r0[tap.z + 1] + w1 * r1[tap.z + 1];
+          const R c2 = w0 * r0[tap.z + 2] + w1 * r1[tap.z + 2];
+          z.x += tap.a0 * c0 + tap.a1 * c1;
+          z.y += tap.b0 * c0 + tap.b1 * c1 + tap.b2 * c2;
+        });
+      } else if (large) {
+        each([&](int n, C &z) {
           R l0, l1;
           cic_pair<R>(large, a.n_low, N, cx, cy, n, l0, l1);
           z.x += l0;
           z.y += l1;
         });
       }
+    }
+    if constexpr (POSVEL) {
+      each([&](int n, C z) {
+        R q0, q1;
+        lattice(n, q0, q1);
+        if constexpr (EXT) {
+          q0 += sh1;
+          q1 += sh1;
+        }
+        pos[n] = C{wrap_box<R>(q0 + z.x, box), wrap_box<R>(q1 + z.y, box)};
+        vel[n] = C{vfac * z.x, vfac * z.y};
+      });
+    } else if constexpr (ONLY_PSI) {
+      each([&](int n, C z) { psi[n] = z; });
+    } else {
       if (psi) {
         if (a.accumulate) {
           each([&](int n, C z) {
@@ -1156,10 +1227,21 @@ cudaError_t ct_launch_dual(const AxisArgs &in, cudaStream_t s) {
 }
 
 template <typename R, int N, int V, bool EXT = false, int OUT = 0>
-cudaError_t ct_launch_zinv(const ZInvArgs &a, cudaStream_t s) {
+cudaError_t ct_launch_zinv(const ZInvArgs &in, cudaStream_t s) {
   using Pol = ct::ZPolicy<R, N, V>;
+  ZInvArgs a = in;
   const size_t dense = (Pol::DENSE * 2 * sizeof(R) + 127) & ~(size_t)127;
-  const size_t smem = 128 + dense + (size_t)Pol::WORK_INV * 2 * sizeof(R);
+  size_t smem = 128 + dense + (size_t)Pol::WORK_INV * 2 * sizeof(R);
+  a.large_rows = 0;
+  if (EXT && a.large) {
+    const int rows = merge_rows<N, Pol::L>(a.n_low);
+    const size_t more = 2 * sizeof(R) + (size_t)(N / 2) * sizeof(MergeTap<R>) + (size_t)rows * (a.n_low + 2) * sizeof(R);
+    // not where the lines would cost a CTA its place (nearly equal grids)
+    if (rows > 0 && (smem + more + 1024) * Pol::MINB_INV <= 228 * 1024) {
+      a.large_rows = rows;
+      smem += more;
+    }
+  }
   auto kern = k_zinv_ct<R, N, V, EXT, OUT>;
   cudaError_t e = set_smem(kern, smem);
   if (e != cudaSuccess) return e;
@@ -1211,9 +1293,11 @@ template <typename R, int... NS> struct CtTable {
   }
   template <int N> static cudaError_t axis_n(const AxisArgs &a, cudaStream_t s) {
     if (!a.fwd && !a.inv) return cudaErrorInvalidValue;
-    if (a.pre && a.qmin > 0) {  // the Sec. 2.4 cut (the fused x pass only): variant 0
+    if (a.pre && a.qmin > 0) {  // the Sec. 2.4 cut (the fused x pass only)
       if (!(a.fwd && a.inv)) return cudaErrorInvalidValue;
-      return ct_launch_axis<R, N, 0, kAxisFwdInv, true>(a, s);
+      constexpr int V = ct::AxisPolicy<R, N, 2>::THREE ? 2 : 0;  // as the plain x pass (488 -> 422 us at 512^3)
+      if (a.interp) return ct_launch_axis<R, N, V, kAxisFwdInv, true, kFiltInterp>(a, s);
+      return ct_launch_axis<R, N, V, kAxisFwdInv, true>(a, s);
     }
     if constexpr (ct::ct_tuned<R>(N)) {
       if (a.variant == 1) return axis_v<N, 1>(a, s);
@@ -1263,8 +1347,13 @@ template <typename R, int... NS> struct CtTable {
                        : ct_launch_zinv<R, N, V, false, kZPosVel>(a, s);
   }
   template <int N> static cudaError_t zinv_n(const ZInvArgs &a, cudaStream_t s) {
-    if (a.large || a.pos2 || a.shift != 0.0 || a.shift2 != 0.0)  // Secs. 2.2, 2.4 options: variant 0
-      return ct_launch_zinv<R, N, 0, true>(a, s);
+    if (a.large || a.pos2 || a.shift != 0.0 || a.shift2 != 0.0){  // Secs. 2.2, 2.4 options: variant 0
+      const bool posvel = a.large && a.pos && a.vel && !a.psi && !a.pos2 && !a.psi_list && !a.pos_list &&
+                          !a.vel_list && !a.accumulate && (a.mul_kz != 0) == (a.comp == 2);
+      if (!posvel) return ct_launch_zinv<R, N, 0, true>(a, s);
+      return a.comp == 2 ? ct_launch_zinv<R, N, 0, true, kZPosVelZ>(a, s)
+                         : ct_launch_zinv<R, N, 0, true, kZPosVel>(a, s);
+    }
     if constexpr (ct::ct_tuned<R>(N)) {
       if (a.variant == 1) return zinv_v<N, 1>(a, s);
       if (a.variant == 2) return zinv_v<N, 2>(a, s);

@@ -166,6 +166,7 @@ struct ZInvArgs {
   // the transform's output before the epilogue; nullptr: none
   const void *large;
   int n_low;
+  int large_rows;         // coarse lines staged per tile (set by the launcher; 0: none)
   // Sec. 2.2 particle options: shift added to q for pos (periodic shift, and
   // the dark-matter offset of gas pairs); pos2: a second position output
   // (the gas partners) with its own shift2; nullptr: none
