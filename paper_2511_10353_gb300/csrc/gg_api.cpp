@@ -104,6 +104,9 @@ struct gg_plan {
   // power spectrum: the grid's shell weights and weighted |m| for shell_nb shells
   std::vector<double> shell_w, shell_m;
   int shell_nb = 0;
+  // set for the duration of a call: the run-time kernels also where N has
+  // specialised ones (run_power_spectrum)
+  bool runtime_kernels = false;
   double *diag = nullptr;  // device sums of the diagnostics, grown on use
   size_t diag_words = 0;
 };
@@ -484,7 +487,7 @@ gg::AxisArgs axis_args(gg_plan_t *plan, int axis, const void *src) {
 template <typename R>
 gg_status launch_axis_timed(gg_plan_t *plan, const gg::AxisArgs &c, int kind, const char *what) {
   const double cb = (double)plan->cells * sizeof(R);
-  const bool spec = gg::spec_has<R>(c.n);
+  const bool spec = gg::spec_has<R>(c.n) && !plan->runtime_kernels;
   const double bytes = (c.fwd && !c.inv ? 2 : 1 + c.nout) * cb;
   cudaError_t e;
   {
@@ -514,7 +517,7 @@ gg_status forward_z(gg_plan_t *plan, uint64_t seed, const void *noise, void *dst
   cudaError_t e;
   {
     ProfScope ps(plan, kZFwd, noise ? 2 * cb : cb);
-    e = gg::spec_has<R>(n) ? gg::spec_zfwd<R>(z, plan->stream) : gg::launch_zfwd<R>(z, plan->stream);
+    e = gg::spec_has<R>(n) && !plan->runtime_kernels ? gg::spec_zfwd<R>(z, plan->stream) : gg::launch_zfwd<R>(z, plan->stream);
   }
   return e == cudaSuccess ? GG_OK : cuda_fail(plan, e, "z forward pass");
 }
@@ -1241,15 +1244,23 @@ gg_status run_power_spectrum(gg_plan_t *plan, const void *field, int nbins, doub
   const int n = (int)plan->p.n;
   gg_status st = ensure_diag(plan, 2 * (size_t)nbins);
   if (st != GG_OK) return st;
-  if ((st = forward_zy<R>(plan, 0, field)) != GG_OK) return st;
-  gg::AxisArgs x = axis_args<R>(plan, 0, plan->work);
-  x.fwd = 1;
-  x.inv = 0;
-  x.nout = 1;
-  x.dst[0] = plan->work;
-  x.mul[0] = gg::kMulNone;
-  x.variant = plan->variant[1];
-  if ((st = launch_axis_timed<R>(plan, x, kXFused, "x forward pass")) != GG_OK) return st;
+  // P(k) is returned in FP64, where another rounding of the FP32 transforms shows
+  // (1e-8): the FP32 sizes whose specialised kernels have one tile shape keep
+  // the run-time kernels' arithmetic here
+  plan->runtime_kernels = sizeof(R) == 4 && !gg::spec_tuned<R>(n);
+  st = forward_zy<R>(plan, 0, field);
+  if (st == GG_OK) {
+    gg::AxisArgs x = axis_args<R>(plan, 0, plan->work);
+    x.fwd = 1;
+    x.inv = 0;
+    x.nout = 1;
+    x.dst[0] = plan->work;
+    x.mul[0] = gg::kMulNone;
+    x.variant = plan->variant[1];
+    st = launch_axis_timed<R>(plan, x, kXFused, "x forward pass");
+  }
+  plan->runtime_kernels = false;
+  if (st != GG_OK) return st;
   double *sums = plan->diag;
   cudaError_t e = cudaSuccess;
   gg::ShellArgs a{};

@@ -1,14 +1,14 @@
 // Sec. 2.1 diagnostics on sm_103a: shell sums of a half spectrum for the
 // power-spectrum estimator, and the moments of a real field.
 //
-// Shell sums: the eight lines (+-m_x, +-m_y) and (+-m_y, +-m_x) of the half
-// spectrum share every |m|, so a warp takes such an orbit, adds the eight
-// |F|^2 of each k_z in registers and makes one shell index and one addition
-// to the CTA's shared-memory sums of them. The grid's sums (weight, weight
-// |m|) are formed once per plan and shell count. Shell index by exact integer
-// arithmetic: b = floor(|m| + 1/2) is the smallest b with 4 m^2 < (2b + 1)^2,
-// from an FP32 estimate (m^2 < 2^24) corrected by one; an FP64 square root a
-// mode had bound the kernel (two FP64 lanes an SM). 512^3: 1375 -> 63 us.
+// Shell sums: warps stride over the (x, y) lines of the half spectrum; the
+// shell index by exact integer arithmetic: b = floor(|m| + 1/2) is the smallest b
+// with 4 m^2 < (2b + 1)^2, from an FP32 estimate (m^2 < 2^24) corrected by one.
+// An FP64 square root a mode had bound the kernel (two FP64 lanes an SM): 512^3
+// 1375 -> 259 us. Adding the eight lines of an orbit (+-m_x, +-m_y) before
+// the shared-memory sums took 63 us, but rounds P(k), which callers get in
+// FP64, differently by 4e-9; the order of the additions is kept instead. The
+// grid's sums (weight, weight |m|) are formed once per plan and shell count.
 //
 // Moments: per-CTA FP64 sum (first pass) or sum of squared deviations
 // (second pass), minimum and maximum, one slot per CTA, added in a fixed
@@ -33,68 +33,94 @@
 namespace gg {
 namespace {
 
-// GEOM: the grid's own sums (weight, weight |m|: FP64, once per plan and
-// shell count); otherwise the power sums alone, accumulated in the field's
-// precision per CTA (A) and in FP64 across CTAs. `copies` (a power of two) of
-// the shell sums per CTA, taken by lane, so that lanes of one shell seldom
-// meet; their stride is odd (other banks).
-template <typename R, typename A, bool GEOM>
-__global__ void __launch_bounds__(256) k_shell_sums(const ShellArgs a, int copies) {
+// Shell of a mode: floor(|m| + 1/2), m2 < 2^24 (exact in FP32).
+__device__ __forceinline__ int shell_of(int m2) {
+  int b = (int)(sqrtf((float)m2) + 0.5f);
+  if ((2 * b + 1) * (2 * b + 1) <= 4 * m2) ++b;
+  if (b > 0 && 4 * m2 < (2 * b - 1) * (2 * b - 1)) --b;
+  return b;
+}
+
+// Power sums: one warp per (x, y) line of the half spectrum at a time, its own
+// copy of the shell sums in shared memory (copies = warps of the CTA, or fewer
+// when the bins are many), accumulated in the field's precision per CTA (A) and
+// in FP64 across CTAs. A line's values are read before the first addition.
+template <typename R, typename A>
+__global__ void __launch_bounds__(256) k_shell_power(const ShellArgs a, int copies) {
   extern __shared__ __align__(16) unsigned char raw[];
-  A *acc = reinterpret_cast<A *>(raw);  // [copies][stride], K nbins used, K = 2 (GEOM) or 1
-  constexpr int K = GEOM ? 2 : 1;
-  const int nb = a.nbins, stride = (K * nb) | 1;
-  for (int i = threadIdx.x; i < copies * stride; i += blockDim.x) acc[i] = (A)0;
+  A *acc = reinterpret_cast<A *>(raw);  // [copies][nbins]
+  const int nb = a.nbins;
+  for (int i = threadIdx.x; i < copies * nb; i += blockDim.x) acc[i] = (A)0;
   __syncthreads();
   const Cx<R> *spec = reinterpret_cast<const Cx<R> *>(a.spec);
   const int n = a.n, half = n / 2;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  A *mine = acc + (lane & (copies - 1)) * stride;
-  // orbits (u, v), 0 <= v <= u < N/2 (|m_j| = N/2 left out; k_z = N/2 is not stored)
-  const int orbits = half * (half + 1) / 2;
-  const int wstep = (int)gridDim.x * (blockDim.x >> 5);
-  for (int o = (int)blockIdx.x * (blockDim.x >> 5) + warp; o < orbits; o += wstep) {
-    int u = (int)((sqrtf(8.0f * (float)o + 1.0f) - 1.0f) * 0.5f);
-    while (u * (u + 1) / 2 > o) --u;
-    while ((u + 1) * (u + 2) / 2 <= o) ++u;
-    const int v = o - u * (u + 1) / 2;
-    // its lines: q bit 0 the sign of the first index, bit 1 of the second, bit 2 swapped
-    const Cx<R> *row[8];
-    int lines = 0;
+  A *mine = acc + (size_t)(warp % copies) * nb;
+  const int lines = n * n, wstep = (int)gridDim.x * (int)(blockDim.x >> 5);
+  for (int line = (int)(blockIdx.x * (blockDim.x >> 5)) + warp; line < lines; line += wstep) {
+    const int x = line / n, y = line - x * n;
+    if (x == half || y == half) continue;  // |m_j| = N/2 left out (k_z = N/2 is not stored)
+    const int mx = x < half ? x : x - n, my = y < half ? y : y - n;
+    const int p2 = mx * mx + my * my;
+    const Cx<R> *row = spec + (int64_t)line * half;
+    constexpr int AHEAD = 8;
+    for (int k0 = 0; k0 < half; k0 += 32 * AHEAD) {
+      if (shell_of(p2 + k0 * k0) >= nb) break;  // the shells grow along the line
+      Cx<R> v[AHEAD];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int p = q & 4 ? v : u, r = q & 4 ? u : v;
-      const bool on = !((q & 1) && p == 0) && !((q & 2) && r == 0) && !((q & 4) && u == v);
-      const int x = (q & 1) ? n - p : p, y = (q & 2) ? n - r : r;
-      row[q] = on ? spec + ((int64_t)x * n + y) * half : nullptr;
-      lines += on ? 1 : 0;
-    }
-    const int p2 = u * u + v * v;
-    for (int kz = lane; kz < half; kz += 32) {
-      const int m2 = p2 + kz * kz;  // < 2^24: exact in FP32
-      int b = (int)(sqrtf((float)m2) + 0.5f);
-      if ((2 * b + 1) * (2 * b + 1) <= 4 * m2) ++b;
-      if (b > 0 && 4 * m2 < (2 * b - 1) * (2 * b - 1)) --b;
-      if (b >= nb) break;  // the shells grow along the line
-      const int w = kz == 0 ? 1 : 2;
-      if constexpr (GEOM) {
-        atomicAdd(&mine[b], (A)(w * lines));
-        atomicAdd(&mine[nb + b], (A)(w * lines) * (A)sqrt((double)m2));
-      } else {
-        Cx<R> f[8];
+      for (int q = 0; q < AHEAD; ++q) {
+        const int kz = k0 + 32 * q + lane;
+        if (kz < half) v[q] = row[kz];
+      }
 #pragma unroll
-        for (int q = 0; q < 8; ++q) f[q] = row[q] ? row[q][kz] : Cx<R>{(R)0, (R)0};
-        A t = (A)0;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) t += f[q].x * f[q].x + f[q].y * f[q].y;
-        atomicAdd(&mine[b], (A)w * t);
+      for (int q = 0; q < AHEAD; ++q) {
+        const int kz = k0 + 32 * q + lane;
+        const int b = shell_of(p2 + kz * kz);
+        if (kz < half && b < nb) atomicAdd(&mine[b], (A)(kz == 0 ? 1 : 2) * (v[q].x * v[q].x + v[q].y * v[q].y));
       }
     }
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < K * nb; i += blockDim.x) {
+  for (int i = threadIdx.x; i < nb; i += blockDim.x) {
     double t = 0.0;
-    for (int c = 0; c < copies; ++c) t += (double)acc[c * stride + i];
+    for (int c = 0; c < copies; ++c) t += (double)acc[(size_t)c * nb + i];
+    if (t != 0.0) atomicAdd(&a.sums[i], t);
+  }
+}
+
+// The grid's own sums (weight, weight |m|: FP64, once per plan and shell
+// count): a warp per orbit (+-u, +-v), (+-v, +-u) of lines, which share every
+// |m|. `copies` of the sums per CTA, taken by lane, at an odd stride.
+__global__ void __launch_bounds__(256) k_shell_grid(const ShellArgs a, int copies) {
+  extern __shared__ __align__(16) unsigned char raw[];
+  double *acc = reinterpret_cast<double *>(raw);  // [copies][stride], 2 nbins used
+  const int nb = a.nbins, stride = (2 * nb) | 1;
+  for (int i = threadIdx.x; i < copies * stride; i += blockDim.x) acc[i] = 0.0;
+  __syncthreads();
+  const int half = a.n / 2;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double *mine = acc + (lane & (copies - 1)) * stride;
+  const int orbits = half * (half + 1) / 2;  // 0 <= v <= u < N/2 (|m_j| = N/2 left out)
+  const int wstep = (int)gridDim.x * (int)(blockDim.x >> 5);
+  for (int o = (int)(blockIdx.x * (blockDim.x >> 5)) + warp; o < orbits; o += wstep) {
+    int u = (int)((sqrtf(8.0f * (float)o + 1.0f) - 1.0f) * 0.5f);
+    while (u * (u + 1) / 2 > o) --u;
+    while ((u + 1) * (u + 2) / 2 <= o) ++u;
+    const int v = o - u * (u + 1) / 2;
+    const int lines = (u ? 2 : 1) * (v ? 2 : 1) * (u != v ? 2 : 1);
+    for (int kz = lane; kz < half; kz += 32) {
+      const int m2 = u * u + v * v + kz * kz;
+      const int b = shell_of(m2);
+      if (b >= nb) break;  // the shells grow along the line
+      const double w = (double)((kz == 0 ? 1 : 2) * lines);
+      atomicAdd(&mine[b], w);
+      atomicAdd(&mine[nb + b], w * sqrt((double)m2));
+    }
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < 2 * nb; i += blockDim.x) {
+    double t = 0.0;
+    for (int c = 0; c < copies; ++c) t += acc[c * stride + i];
     if (t != 0.0) atomicAdd(&a.sums[i], t);
   }
 }
@@ -276,23 +302,29 @@ int grid_for(int64_t work, int per_sm) {
 
 }  // namespace
 
-template <typename R, typename A, bool GEOM> cudaError_t shell_launch(const ShellArgs &a, cudaStream_t s) {
-  const size_t per_copy = (size_t)((GEOM ? 2 : 1) * a.nbins | 1) * sizeof(A);
-  int copies = 8;
-  while (copies > 1 && copies * per_copy > 48 * 1024) copies /= 2;
+template <typename K> cudaError_t shell_launch(K kern, const ShellArgs &a, int copies, size_t per_copy, int blocks,
+                                               cudaStream_t s) {
   const size_t smem = per_copy * copies;
-  auto kern = k_shell_sums<R, A, GEOM>;
   if (smem > 48 * 1024) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  const int64_t half = a.n / 2;
-  kern<<<grid_for(half * (half + 1) / 2 * 32, 4), 256, smem, s>>>(a, copies);
+  kern<<<blocks, 256, smem, s>>>(a, copies);
   return cudaGetLastError();
 }
 
 template <typename R> cudaError_t launch_shell_sums(const ShellArgs &a, bool geometry, cudaStream_t s) {
-  return geometry ? shell_launch<R, double, true>(a, s) : shell_launch<R, R, false>(a, s);
+  if (geometry) {
+    const size_t per_copy = (size_t)((2 * a.nbins) | 1) * sizeof(double);
+    int copies = 8;
+    while (copies > 1 && copies * per_copy > 48 * 1024) copies /= 2;
+    const int64_t half = a.n / 2;
+    return shell_launch(k_shell_grid, a, copies, per_copy, grid_for(half * (half + 1) / 2 * 32, 4), s);
+  }
+  const size_t per_copy = (size_t)a.nbins * sizeof(R);
+  int copies = (int)((192 * 1024) / per_copy);
+  copies = copies > 8 ? 8 : (copies < 1 ? 1 : copies);
+  return shell_launch(k_shell_power<R, R>, a, copies, per_copy, grid_for((int64_t)a.n * a.n * 32 / 8, 2), s);
 }
 
 template <typename R> int moment_blocks(int64_t count) {
