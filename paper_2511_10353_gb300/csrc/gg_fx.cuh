@@ -120,7 +120,7 @@ struct Weight {
   int c;
   bool neg;
 };
-__device__ __forceinline__ Weight weight_one() { return Weight{1u << 9, 9, false}; }
+__device__ __forceinline__ Weight weight_one() { return Weight{1u << 10, 10, false}; }
 __device__ __forceinline__ Weight weight_int(int f) {  // |f| < 2^11
   const uint32_t a = (uint32_t)(f < 0 ? -f : f);
   const int c = a ? __clz(a) - 21 : 0;
@@ -132,9 +132,11 @@ __device__ __forceinline__ long long to_fixed(double v, const Scale &sc, const W
   const uint32_t mh = (hi & 0xfffffu) | 0x100000u;
   const unsigned long long p = (unsigned long long)lo * w.m;
   const unsigned long long m = p + ((unsigned long long)(mh * w.m) << 32);
-  int r = sc.k + w.c - e;
+  // m >= 2^62 and the result is below 2^62: r >= 1. Rounded to nearest: cutting
+  // off would shrink every transform by up to 2^-53.
+  int r = sc.k + w.c - e - 1;
   r = r < 63 ? r : 63;
-  unsigned long long f = m >> r;
+  unsigned long long f = ((m >> r) + 1) >> 1;
   if (e == 0) f = 0;  // zeros and subnormals
   const long long g = (long long)f;
   return ((int)hi < 0) != w.neg ? -g : g;
