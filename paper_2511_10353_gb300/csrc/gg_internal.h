@@ -318,6 +318,12 @@ bool persist_has(int n);
 // Fills the tile shapes and tensor maps and launches on s (capturable).
 cudaError_t launch_persist(PersistPlan p, cudaStream_t s, int *launched_blocks);
 
+// CTAs of a kernel that fill the current device (SMs times CTAs an SM). The
+// occupancy query costs more than a microsecond a launch, as much as the
+// launch itself, and its answer is a property of the kernel, the shape and the
+// device: asked once for each (a few hundred entries at most; any thread).
+int resident_blocks(const void *kernel, int threads, size_t smem);
+
 // Message returned by gg_last_error(NULL) on this host thread.
 void set_thread_error(const char *msg);
 cudaError_t launch_noise_bits(uint64_t seed, int64_t first, int64_t count, uint32_t *out,

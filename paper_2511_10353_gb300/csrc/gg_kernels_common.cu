@@ -1,4 +1,9 @@
-// Precision-independent kernels and helpers: raw Philox words, tile sizes.
+// Precision-independent kernels and helpers: raw Philox words, tile sizes,
+// grid sizes.
+#include <map>
+#include <mutex>
+#include <tuple>
+
 #include "gg_device.cuh"
 
 namespace gg {
@@ -18,6 +23,26 @@ cudaError_t launch_noise_bits(uint64_t seed, int64_t first, int64_t count, uint3
   k_noise_bits<<<(unsigned)blocks, threads, 0, s>>>(seed, first, count,
                                                      reinterpret_cast<uint4 *>(out));
   return cudaGetLastError();
+}
+
+int resident_blocks(const void *kernel, int threads, size_t smem) {
+  static std::mutex mu;
+  static std::map<std::tuple<const void *, int, int, size_t>, int> known;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  const auto key = std::make_tuple(kernel, dev, threads, smem);
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    const auto it = known.find(key);
+    if (it != known.end()) return it->second;
+  }
+  int sms = 0, per = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem) != cudaSuccess || per < 1)
+    return sms;  // not kept: the launch will tell
+  std::lock_guard<std::mutex> lock(mu);
+  known[key] = sms * per;
+  return sms * per;
 }
 
 size_t zpass_smem_bytes(int half_len, int lines, size_t complex_bytes) {

@@ -76,13 +76,7 @@ static cudaError_t make_map(CUtensorMap *m, const AxisArgs &a) {
 
 template <typename K>
 static int persistent_blocks(K kernel, int threads, size_t smem, int64_t tiles) {
-  int dev = 0, sms = 0, per = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem) != cudaSuccess ||
-      per < 1)
-    per = 1;
-  const int64_t b = (int64_t)sms * per;
+  const int64_t b = resident_blocks(reinterpret_cast<const void *>(kernel), threads, smem);
   return (int)(tiles < b ? tiles : b);
 }
 
