@@ -381,14 +381,15 @@ void choose_tiles(gg_plan_t *plan) {
 // taken, one realization each:
 // * z passes: warp barriers, with half the lines per CTA up to N = 256
 //   (N = 128: 12.4 + 35.5 -> 11.5 + 31.6; 256: 49.5 + 123.5 -> 46.0 + 119.7) and
-//   all of them above (384: 157.9 + 357 -> 147.6 + 356; 512: 336 + 784 -> 310 +
+//   all of them above (384: 157.9 + 357 -> 148.0 + 356; 512: 336 + 784 -> 310 +
 //   775; 1536: 9849 + 21987 -> 9639 + 21844);
-// * x fused: the small tile where three of its CTAs fit an SM (512: 456 -> 420);
-// * y inverses: the small tile, two CTAs an SM, between 256 and 512 (384: 90 +
-//   150 -> 79 + 119); at 512 the two-output one alone, by variant 1 (272 ->
-//   261); elsewhere variant 0 is within 3% of the best.
+// * x fused: the small tile where three of its CTAs fit an SM (384: 240 -> 210;
+//   512: 456 -> 420);
+// * y inverses from 384: the two-output one by variant 1 (384: 150 -> 128; 512:
+//   272 -> 261), the other by variant 1 at 384 (90 -> 79); elsewhere variant 0 is
+//   within 3% of the best.
 // * chunk-major spectra where a row of the x pass's tiles is 2 MB (a memory
-//   page) or more from the next: 768: 7953 -> 7917; 1024: 23050 -> 21640; 1536:
+//   page) or more from the next: 768: 7953 -> 7917; 1024: 22670 -> 21080; 1536:
 //   69980 -> 66990 a run (512, rows of 1 MB: 2191 -> 2178, but its x pass's tile
 //   is narrower than the others').
 void default_shapes(gg_plan_t *plan) {
@@ -398,9 +399,8 @@ void default_shapes(gg_plan_t *plan) {
   if (!gg::spec_tuned<float>(n)) return;
   plan->variant[0] = plan->variant[5] = n <= 256 ? 3 : 2;
   plan->variant[2] = gg::spec_three_ctas<float>(n) ? 2 : 0;
-  const bool mid = n > 256 && n < 512;
-  plan->variant[3] = mid ? 2 : 0;
-  plan->variant[4] = mid ? 2 : (n == 512 ? 1 : 0);
+  plan->variant[3] = n > 256 && n < 512 ? 1 : 0;
+  plan->variant[4] = n > 256 && n <= 512 ? 1 : 0;
 }
 
 void release(gg_plan_t *plan) {
@@ -2134,9 +2134,11 @@ gg_status gg_batch_plan(gg_batch_t **batch, const gg_params *params, int count, 
   for (auto &g : b->groups) {
     const gg_params &p = params[g.members[0]];
     if ((st = gg_plan(&g.plan, &p, stream)) != GG_OK) break;
-    // several realizations a launch, groups side by side: variant 0 throughout
-    // (16 realizations of 128 .. 384: 5.58 ms, 5.64 with a lone run's choice)
-    for (int &v : g.plan->variant) v = 0;
+    // several realizations a launch, groups side by side: variant 0 but for the
+    // x pass (16 realizations of 128 .. 384: 5.43 ms, 5.58 with variant 0 there too; 5.64 with a lone run's z
+    // passes and y inverses)
+    for (int k = 0; k < 6; ++k)
+      if (k != 2) g.plan->variant[k] = 0;
     const size_t nb = g.members.size();
     const size_t bytes = (size_t)p.n * p.n * p.n * (p.prec == GG_F64 ? 8 : 4) * nb;
     for (void *&w : g.work)

@@ -14,6 +14,17 @@
 #include "gg_fx.cuh"
 
 namespace gg {
+
+// FP32 with schedules of their own for the z lines (see LineT)
+struct Line512 {
+  float v;
+};
+struct Line384 {
+  float v;
+};
+template <> struct CxOf<Line512> { using T = float2; };
+template <> struct CxOf<Line384> { using T = float2; };
+
 namespace ct {
 
 // ------------------------------------------------------------ schedules
@@ -26,8 +37,10 @@ namespace ct {
 // pipe, not the stage count), use radix 8 first, then 4 or 2, then the 3s.
 // The fixed-point codelets of the FP64 sizes (kFx, R = long long) keep a thread
 // at 8 or 12 elements (four registers each) where the length allows it.
-constexpr int kBig = 1 << 20, kFx = 1 << 21;
+constexpr int kBig = 1 << 20, kFx = 1 << 21, kLine = 1 << 22;
 template <typename R> __host__ __device__ constexpr int skey(int n) {
+  if (std::is_same<R, Line512>::value) return n | kLine;
+  if (std::is_same<R, Line384>::value) return n;
   return sizeof(R) == 4 ? (n | kBig) : (std::is_same<R, long long>::value ? (n | kFx) : n);
 }
 __host__ __device__ constexpr int key_n(int key) { return key & (kBig - 1); }
@@ -57,6 +70,7 @@ __host__ __device__ constexpr int big_radix(int n, int s) {
     case 216: return s < 3 ? 6 : 0;
     case 288: return s == 0 ? 12 : (s == 1 ? 24 : 0);
     case 324: return s < 2 ? 6 : (s == 2 ? 9 : 0);
+    case 384: return s < 2 ? 8 : (s == 2 ? 6 : 0);
     case 432: return s < 2 ? 6 : (s == 2 ? 12 : 0);
     case 576: return s < 2 ? 24 : 0;
     case 648: return s < 2 ? 6 : (s == 2 ? 18 : 0);
@@ -88,6 +102,7 @@ __host__ __device__ constexpr int fx_radix(int n, int s) {
   }
 }
 __host__ __device__ constexpr int own_radix(int key, int s) {
+  if (key & kLine) return s < 2 ? 16 : (s == 2 ? 2 : 0);
   return (key & kBig) ? big_radix(key_n(key), s) : ((key & kFx) ? fx_radix(key_n(key), s) : 0);
 }
 __host__ __device__ constexpr bool is_big(int key) { return own_radix(key, 0) != 0; }
@@ -599,13 +614,13 @@ template <typename R, int N, int V> struct AxisPolicy {
   // pass may still keep that pass at one); variant 1 of the large radices:
   // as many CTAs as the tiles' shared memory allows, up to three
   static constexpr int SMEM_EST = 128 + 2 * N * B * CB;
-  // variant 2 of the FP32 large radices from N = 512, where the two tiles
+  // variant 2 of the FP32 large radices from N = 384, where the two tiles
   // and the largest filter table of three CTAs fit an SM: three CTAs with
   // the spectrum in registers (the outputs leave by TMA from the tile buffer
   // itself, the twiddles stay in global memory). 512^3 x pass 0.454 ->
-  // 0.421 ms; at N = 256 the two-CTA staging-tile form stays (the batched
+  // 0.421 ms, 384^3 238 -> 210 us; at N = 256 the two-CTA staging-tile form stays (the batched
   // workload measured 17.0 against 17.4 ms with three CTAs there too)
-  static constexpr bool THREE = V == 2 && BIG && sizeof(R) == 4 && N >= 512 &&
+  static constexpr bool THREE = V == 2 && BIG && sizeof(R) == 4 && N >= 384 &&
                                 3 * (SMEM_EST + 4 * kInterpExact + 16 * kMaxInterpCells(N) + 1024) <=
                                     228 * 1024;
   static constexpr int REG_NEED = 4 * E * ((int)sizeof(R) / 4) + 48;
@@ -655,6 +670,16 @@ template <typename R, int N, int V> struct AxisPolicy {
   }
 };
 
+// Stage arithmetic of a z pass's lines of M complex values: lines of 512 (N =
+// 1024) take the schedule 16 x 16 x 2 (Line512), 16 elements a thread and twice
+// the warps of the strided passes' 32 x 16 (1024^3 z forward 3.30 -> 3.02 ms, three
+// z inverses 7.72 -> 7.48), lines of 384 (N = 768) 8 x 8 x 2 x 3 with the last two in
+// registers (Line384; three z inverses 2.84 ms, 3.12 with the strided 8 x 8 x 6).
+template <typename R, int M>
+using LineT = typename std::conditional<
+    sizeof(R) == 4 && M == 512, Line512,
+    typename std::conditional<sizeof(R) == 4 && M == 384, Line384, R>::type>::type;
+
 // z passes: lines per tile, variant 0 ~256 threads (sized so that two dense
 // tiles and a padded tile fit in 160 KB), variant 1 half as many lines,
 // variant 2 the lines of variant 0 with warp instead of CTA barriers between
@@ -662,12 +687,13 @@ template <typename R, int N, int V> struct AxisPolicy {
 // variant 3 the lines of variant 1 with warp barriers.
 template <typename R, int N, int V> struct ZPolicy {
   static constexpr int M = N / 2;
-  static constexpr int E = elems(skey<R>(M));
+  using T = LineT<R, M>;  // the lines' stage arithmetic
+  static constexpr int E = elems(skey<T>(M));
   static constexpr int P = M / E;
   static constexpr int CB = 2 * (int)sizeof(R);
   static constexpr int LD = M + (M >> 4) + 1;  // tile sizing (the widest padding)
   // the forward's last two and the inverse's first two stages in registers
-  static constexpr bool FUSE = fuse_pair<R, M, E>();
+  static constexpr bool FUSE = fuse_pair<T, M, E>();
   // Padding of the work tile, per direction: one empty slot every PAD values
   // (0: none). Chosen by counting the shared-memory wavefronts of every
   // stage's stores and loads for each size; FP32 (FP64 keeps 1 in 16).

@@ -676,7 +676,8 @@ __device__ __forceinline__ bool zinv_body(const ZInvArgs &a, int64_t t0, int64_t
   using C = Cx<R>;
   using Pol = ct::ZPolicy<R, N, V>;
   constexpr int M = Pol::M, E = Pol::E, P = Pol::P, L = Pol::L, LD = Pol::LD_INV, PAD = Pol::PAD_INV;
-  constexpr int KM = ct::skey<R>(M);
+  using LT = typename Pol::T;
+  constexpr int KM = ct::skey<LT>(M);
   constexpr int S = ct::nstages(KM);
   constexpr int RL = ct::radix_of(KM, S - 1, true), SPANL = M / RL, NBL = E / RL;
   // stages of the inverse done in registers straight from the c2r
@@ -783,8 +784,8 @@ __device__ __forceinline__ bool zinv_body(const ZInvArgs &a, int64_t t0, int64_t
       }
     }
     if constexpr (HEAD == 2) {  // the inverse's first two stages in registers
-      ct::inverse_head_regs<R, M, E>(tw_half, v);
-      ct::inverse_head_store<R, M, E>(p, v, st_w);
+      ct::inverse_head_regs<LT, M, E>(tw_half, v);
+      ct::inverse_head_store<LT, M, E>(p, v, st_w);
     } else if constexpr (HEAD == 1) {  // the first stage (no twiddles: NS = 1) in registers
       constexpr int RA = ct::radix_of(KM, 0, true), NBA = E / RA;
 #pragma unroll
@@ -799,8 +800,8 @@ __device__ __forceinline__ bool zinv_body(const ZInvArgs &a, int64_t t0, int64_t
       fence_proxy_async_smem();
       issue(tn);
     }
-    ct::stages<R, M, E, true, HEAD, S - 1, Pol::SY | ct::kNoRangeHint>(p, tw_half, ld_w, st_w);
-    ct::last_stage_regs<R, M, E, true, false>(p, tw_half, ld_w, v);
+    ct::stages<LT, M, E, true, HEAD, S - 1, Pol::SY | ct::kNoRangeHint>(p, tw_half, ld_w, st_w);
+    ct::last_stage_regs<LT, M, E, true, false>(p, tw_half, ld_w, v);
     // line -> (realization, x, y): line counts stay below 2^32 (N <= 4096, the
     // host bounds the batch), so 32-bit divisions suffice
     const uint32_t line = (uint32_t)(t * L + l);
@@ -930,7 +931,8 @@ __device__ __forceinline__ bool zfwd_body(const ZFwdArgs &a, int64_t t0, int64_t
   using C = Cx<R>;
   using Pol = ct::ZPolicy<R, N, V>;
   constexpr int M = Pol::M, E = Pol::E, P = Pol::P, L = Pol::L, LD = Pol::LD_FWD, PAD = Pol::PAD_FWD;
-  constexpr int KM = ct::skey<R>(M);
+  using LT = typename Pol::T;
+  constexpr int KM = ct::skey<LT>(M);
   constexpr int S = ct::nstages(KM);
   constexpr int DENSE_STRIDE = (int)(((Pol::DENSE * sizeof(C) + 127) / 128) * 128 / sizeof(C));
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -970,7 +972,7 @@ __device__ __forceinline__ bool zfwd_body(const ZFwdArgs &a, int64_t t0, int64_t
       phase ^= 1;
       const C *dl = dense + l * M;
       auto ld_d = [&](int n) { return dl[n]; };
-      ct::stage<R, M, E, 0, false, ct::kSyncNone>(p, tw_half, ld_d, st_w);
+      ct::stage<LT, M, E, 0, false, ct::kSyncNone>(p, tw_half, ld_d, st_w);
       __syncthreads();
       if (tid == 0 && t + tstep < tlimit) {  // the dense tile has been read: fetch the next block
         fence_proxy_async_smem();
@@ -1000,10 +1002,10 @@ __device__ __forceinline__ bool zfwd_body(const ZFwdArgs &a, int64_t t0, int64_t
       ct::stage_barrier<Pol::SY>();
     }
     if constexpr (Pol::FUSE) {  // the last two stages in registers, stored in natural order
-      ct::stages<R, M, E, false, FIRST, S - 2, Pol::SY>(p, tw_half, ld_w, st_w);
+      ct::stages<LT, M, E, false, FIRST, S - 2, Pol::SY>(p, tw_half, ld_w, st_w);
       constexpr int RB = ct::radix_of(KM, S - 1, false), NBB = E / RB, SPANB = M / RB;
       C v[E];
-      ct::last_two_stages_regs<R, M, E>(p, tw_half, ld_w, v);
+      ct::last_two_stages_regs<LT, M, E>(p, tw_half, ld_w, v);
       ct::stage_barrier<Pol::SY>();
 #pragma unroll
       for (int b = 0; b < NBB; ++b)
@@ -1011,7 +1013,7 @@ __device__ __forceinline__ bool zfwd_body(const ZFwdArgs &a, int64_t t0, int64_t
         for (int r = 0; r < RB; ++r) st_w(p + P * b + r * SPANB, v[b * RB + r]);
       ct::stage_barrier<Pol::SY>();
     } else {
-      ct::stages<R, M, E, false, FIRST, S, Pol::SY>(p, tw_half, ld_w, st_w);
+      ct::stages<LT, M, E, false, FIRST, S, Pol::SY>(p, tw_half, ld_w, st_w);
     }
     // X_k = S/2 + D u_k with S = Z_k + conj Z_{M-k}, D = Z_k - conj Z_{M-k},
     // u_k = -(i/2) w_k; the partner X_{M-k} = conj(S/2 - D u_k) (w_{M-k} =
@@ -1063,7 +1065,8 @@ __global__ void __launch_bounds__(ct::ZPolicy<R, N, 0>::THREADS, ct::ZPolicy<R, 
   using C = Cx<R>;
   using Pol = ct::ZPolicy<R, N, 0>;
   constexpr int M = Pol::M, E = Pol::E, P = Pol::P, L = Pol::L, LD = Pol::LD_FWD, PAD = Pol::PAD_FWD;
-  constexpr int KM = ct::skey<R>(M);
+  using LT = typename Pol::T;
+  constexpr int KM = ct::skey<LT>(M);
   constexpr int S = ct::nstages(KM);
   constexpr int RL = ct::radix_of(KM, S - 1, true), SPANL = M / RL, NBL = E / RL;
   constexpr int DENSE_STRIDE = (int)(((Pol::DENSE * sizeof(C) + 127) / 128) * 128 / sizeof(C));
@@ -1098,13 +1101,13 @@ __global__ void __launch_bounds__(ct::ZPolicy<R, N, 0>::THREADS, ct::ZPolicy<R, 
     auto ld_d = [&](int n) { return dl[n]; };
     auto ld_w = [&](int n) { return work[zpad<LD, PAD>(l, n)]; };
     auto st_w = [&](int n, C v) { work[zpad<LD, PAD>(l, n)] = v; };
-    ct::stage<R, M, E, 0, false, ct::kSyncNone>(p, tw_half, ld_d, st_w);
+    ct::stage<LT, M, E, 0, false, ct::kSyncNone>(p, tw_half, ld_d, st_w);
     __syncthreads();
     if (tid == 0 && t + gridDim.x < ntiles) {  // the dense tile has been read
       fence_proxy_async_smem();
       issue(t + gridDim.x);
     }
-    ct::stages<R, M, E, false, 1, S, ct::kSyncCta>(p, tw_half, ld_w, st_w);
+    ct::stages<LT, M, E, false, 1, S, ct::kSyncCta>(p, tw_half, ld_w, st_w);
     static_assert(P * (E / 2) == M / 2, "conjugate pairs");
 #pragma unroll
     for (int i = 0; i < E / 2; ++i) {  // both members of a pair in one thread, in place
@@ -1132,9 +1135,9 @@ __global__ void __launch_bounds__(ct::ZPolicy<R, N, 0>::THREADS, ct::ZPolicy<R, 
       }
     }
     __syncthreads();
-    ct::stages<R, M, E, true, 0, S - 1, ct::kSyncCta>(p, tw_half, ld_w, st_w);
+    ct::stages<LT, M, E, true, 0, S - 1, ct::kSyncCta>(p, tw_half, ld_w, st_w);
     C v[E];
-    ct::last_stage_regs<R, M, E, true>(p, tw_half, ld_w, v);
+    ct::last_stage_regs<LT, M, E, true>(p, tw_half, ld_w, v);
     C *dst = reinterpret_cast<C *>(a.dst) + (t * L + l) * M;
 #pragma unroll
     for (int b = 0; b < NBL; ++b)
