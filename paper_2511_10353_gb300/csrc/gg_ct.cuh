@@ -738,6 +738,13 @@ template <typename R, int N, int V> struct ZPolicy {
   static constexpr int MINB_INV = min_blocks(128 + DENSE * CB + WORK_INV * CB);
   static constexpr int MINB_FWD = min_blocks(WORK_FWD * CB);
   static constexpr int MINB_NOISE = min_blocks(128 + DENSE * CB + WORK_FWD * CB);
+  // the separable filter's pass (two transforms a line, bound by their latency):
+  // 24 warps an SM (512^3 279 -> 273 us)
+  static constexpr int filter_blocks() {
+    const int by_smem = (228 * 1024) / (128 + DENSE * CB + WORK_FWD * CB + 1024), by_warps = 768 / THREADS;
+    const int m = by_smem < by_warps ? by_smem : by_warps;
+    return m < 1 ? 1 : m;
+  }
 };
 
 }  // namespace ct

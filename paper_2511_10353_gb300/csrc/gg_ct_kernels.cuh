@@ -1060,7 +1060,7 @@ __global__ void __launch_bounds__(ct::ZPolicy<R, N, V>::THREADS,
 // registers: with X'_k = F_k X_k, S = X'_k + conj X'_{M-k}, D = X'_k - conj
 // X'_{M-k} and T = i D conj w_k, Z'_k = S + T and Z'_{M-k} = conj(S - T).
 template <typename R, int N>
-__global__ void __launch_bounds__(ct::ZPolicy<R, N, 0>::THREADS, ct::ZPolicy<R, N, 0>::MINB_NOISE)
+__global__ void __launch_bounds__(ct::ZPolicy<R, N, 0>::THREADS, ct::ZPolicy<R, N, 0>::filter_blocks())
     k_zfilter(const ZFilterArgs a) {
   using C = Cx<R>;
   using Pol = ct::ZPolicy<R, N, 0>;
