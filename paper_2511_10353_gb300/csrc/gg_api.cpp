@@ -70,6 +70,9 @@ struct gg_plan {
   // 0 z forward, 1 y forward, 2 x fused, 3 y inverse (x branch),
   // 4 y inverse (y/z branches), 5 z inverse
   int variant[6] = {0, 0, 0, 0, 0, 0};
+  // the passes of a call overlap their launches (default_shapes); the batched
+  // form's do not: its groups run on several streams and are captured
+  int overlap = 0;
   int chunked = 0;  // 1: the three-component chain keeps the spectrum chunk-major (gg_plan_set_layout)
   // fault test (gg_test_arm_fault): the next y forward pass issues no copies
   int test_skip_copy = 0;
@@ -392,8 +395,14 @@ void choose_tiles(gg_plan_t *plan) {
 //   page) or more from the next: 768: 7953 -> 7917; 1024: 22670 -> 21080; 1536:
 //   69980 -> 66990 a run (512, rows of 1 MB: 2191 -> 2178, but its x pass's tile
 //   is narrower than the others').
+// * overlapped launches (short passes only, launch_pass) except for FP64 above
+//   N = 64, where the next pass's CTAs crowd onto the SMs that empty first and
+//   the integer pipes of the others idle (a run, FP64: 32: 84 -> 75; 64: 90.5 ->
+//   85.5; 96: 165 -> 188; 192: 811 -> 857; FP32: 32: 43 -> 33; 64: 43 -> 33; 96:
+//   56 -> 52; 144: 101 -> 90; 216: 261 -> 243; 256: 292 -> 277).
 void default_shapes(gg_plan_t *plan) {
   const int n = (int)plan->p.n;
+  plan->overlap = plan->real_bytes == 4 || n <= 64;
   if (plan->real_bytes != 4 || !gg::spec_has<float>(n)) return;
   plan->chunked = (int64_t)n * (n / 2) * 8 >= ((int64_t)2 << 20);
   if (!gg::spec_tuned<float>(n)) return;
@@ -478,6 +487,7 @@ gg::AxisArgs axis_args(gg_plan_t *plan, int axis, const void *src) {
   c.tw = plan->tab.tw_n;
   c.e = plan->col_e;
   c.rows_box = plan->col_rows_box;
+  c.overlap = plan->overlap;
   c.err = plan->err;
   return c;
 }
@@ -513,6 +523,7 @@ gg_status forward_z(gg_plan_t *plan, uint64_t seed, const void *noise, void *dst
   z.tw_full = plan->tab.tw_n;
   z.variant = plan->variant[0];
   z.err = plan->err;
+  z.overlap = plan->overlap;
   const double cb = (double)plan->cells * sizeof(R);
   cudaError_t e;
   {
@@ -572,6 +583,7 @@ gg_status zinv_pass(gg_plan_t *plan, int comp, const void *src, void *psi, void 
   z.tw_full = plan->tab.tw_n;
   z.err = plan->err;
   z.variant = plan->variant[5];
+  z.overlap = plan->overlap;
   z.large = plan->merge_large[comp];
   z.n_low = plan->merge_nlow;
   {  // Sec. 2.2: shift, and the gas pairs' offsets of half a cell per axis
@@ -1116,6 +1128,7 @@ gg_status run_separable(gg_plan_t *plan, const void *factor, const void *in, voi
   z.tw_half = plan->tab.tw_half;
   z.tw_full = plan->tab.tw_n;
   z.err = plan->err;
+  z.overlap = plan->overlap;
   cudaError_t e;
   {
     ProfScope ps(plan, kZFwd, 2 * cb);
@@ -2139,6 +2152,7 @@ gg_status gg_batch_plan(gg_batch_t **batch, const gg_params *params, int count, 
     // passes and y inverses)
     for (int k = 0; k < 6; ++k)
       if (k != 2) g.plan->variant[k] = 0;
+    g.plan->overlap = 0;
     const size_t nb = g.members.size();
     const size_t bytes = (size_t)p.n * p.n * p.n * (p.prec == GG_F64 ? 8 : 4) * nb;
     for (void *&w : g.work)

@@ -1,7 +1,7 @@
 // Size-specialised kernels of the three transform passes (see gg_ct.cuh).
-// Included by gg_ct_f32.cu / gg_ct_f64.cu, which instantiate them for the
-// grid sizes of the named workloads; every other size runs the run-time
-// kernels of gg_kernels.cuh.
+// Included by gg_ct*_f32.cu, which instantiate them for FP32 (FP64:
+// gg_fx_kernels.cuh); every other size runs the run-time kernels of
+// gg_kernels.cuh.
 #pragma once
 
 #include "gg_ct.cuh"
@@ -434,6 +434,7 @@ template <typename R, int N, int V, int MODE, bool CUT = false, int FILT = kFilt
 __global__ void __launch_bounds__(ct::AxisPolicy<R, N, V>::THREADS, ct::AxisPolicy<R, N, V>::MINB)
     k_axis_ct(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap smap0,
               const __grid_constant__ CUtensorMap smap1, const AxisArgs a) {
+  pass_begin();
   axis_body<R, N, V, MODE, CUT, FILT>(map, a, blockIdx.x, gridDim.x, INT64_MAX, &smap0, &smap1);
 }
 
@@ -455,6 +456,7 @@ template <typename R, int N, int DUAL>
 __global__ void __launch_bounds__(DualPolicy<R, N>::THREADS, DualPolicy<R, N>::MINB)
     k_axis_dual(const __grid_constant__ CUtensorMap map0, const __grid_constant__ CUtensorMap map1,
                 const __grid_constant__ CUtensorMap smap, const AxisArgs a) {
+  pass_begin();
   using C = Cx<R>;
   using Pol = DualPolicy<R, N>;
   constexpr int K = ct::skey<R>(N);
@@ -913,6 +915,7 @@ __device__ __forceinline__ bool zinv_body(const ZInvArgs &a, int64_t t0, int64_t
 template <typename R, int N, int V, bool EXT = false, int OUT = 0>
 __global__ void __launch_bounds__(ct::ZPolicy<R, N, V>::THREADS, ct::ZPolicy<R, N, V>::MINB_INV)
     k_zinv_ct(const ZInvArgs a) {
+  pass_begin();
   zinv_body<R, N, V, EXT, OUT>(a, blockIdx.x, gridDim.x, INT64_MAX);
 }
 
@@ -1050,6 +1053,7 @@ template <typename R, int N, int V, bool NOISE>
 __global__ void __launch_bounds__(ct::ZPolicy<R, N, V>::THREADS,
                                   NOISE ? ct::ZPolicy<R, N, V>::MINB_NOISE : ct::ZPolicy<R, N, V>::MINB_FWD)
     k_zfwd_ct(const ZFwdArgs a) {
+  pass_begin();
   zfwd_body<R, N, V, NOISE>(a, blockIdx.x, gridDim.x, INT64_MAX);
 }
 
@@ -1062,6 +1066,7 @@ __global__ void __launch_bounds__(ct::ZPolicy<R, N, V>::THREADS,
 template <typename R, int N>
 __global__ void __launch_bounds__(ct::ZPolicy<R, N, 0>::THREADS, ct::ZPolicy<R, N, 0>::filter_blocks())
     k_zfilter(const ZFilterArgs a) {
+  pass_begin();
   using C = Cx<R>;
   using Pol = ct::ZPolicy<R, N, 0>;
   constexpr int M = Pol::M, E = Pol::E, P = Pol::P, L = Pol::L, LD = Pol::LD_FWD, PAD = Pol::PAD_FWD;
@@ -1155,8 +1160,7 @@ template <typename R, int N> cudaError_t ct_launch_zfilter(const ZFilterArgs &a,
   auto kern = k_zfilter<R, N>;
   cudaError_t e = set_smem(kern, smem);
   if (e != cudaSuccess) return e;
-  kern<<<persistent_blocks(kern, Pol::THREADS, smem, a.nlines / Pol::L), Pol::THREADS, smem, s>>>(a);
-  return cudaGetLastError();
+  return launch_pass(kern, a.nlines / Pol::L, Pol::THREADS, smem, s, a.overlap, a);
 }
 
 template <typename R, int N, int V, int MODE, bool CUT = false, int FILT = kFiltArgs>
@@ -1196,8 +1200,7 @@ cudaError_t ct_launch_axis(const AxisArgs &in, cudaStream_t s) {
   auto kern = k_axis_ct<R, N, V, MODE, CUT, FILT>;
   if ((e = set_smem(kern, smem)) != cudaSuccess) return e;
   const int64_t tiles = (int64_t)N * a.inner_chunks * (a.nbatch > 0 ? a.nbatch : 1);
-  kern<<<persistent_blocks(kern, Pol::THREADS, smem, tiles), Pol::THREADS, smem, s>>>(map, smap[0], smap[1], a);
-  return cudaGetLastError();
+  return launch_pass(kern, tiles, Pol::THREADS, smem, s, a.overlap, map, smap[0], smap[1], a);
 }
 
 template <typename R, int N, int DUAL>
@@ -1225,8 +1228,7 @@ cudaError_t ct_launch_dual(const AxisArgs &in, cudaStream_t s) {
   auto kern = k_axis_dual<R, N, DUAL>;
   if ((e = set_smem(kern, smem)) != cudaSuccess) return e;
   const int64_t tiles = (int64_t)N * ((N / 2) / Pol::B);
-  kern<<<persistent_blocks(kern, Pol::THREADS, smem, tiles), Pol::THREADS, smem, s>>>(map[0], map[1], map[2], a);
-  return cudaGetLastError();
+  return launch_pass(kern, tiles, Pol::THREADS, smem, s, a.overlap, map[0], map[1], map[2], a);
 }
 
 template <typename R, int N, int V, bool EXT = false, int OUT = 0>
@@ -1248,8 +1250,7 @@ cudaError_t ct_launch_zinv(const ZInvArgs &in, cudaStream_t s) {
   auto kern = k_zinv_ct<R, N, V, EXT, OUT>;
   cudaError_t e = set_smem(kern, smem);
   if (e != cudaSuccess) return e;
-  kern<<<persistent_blocks(kern, Pol::THREADS, smem, a.nlines / Pol::L), Pol::THREADS, smem, s>>>(a);
-  return cudaGetLastError();
+  return launch_pass(kern, a.nlines / Pol::L, Pol::THREADS, smem, s, a.overlap, a);
 }
 
 template <typename R, int N, int V, bool NOISE>
@@ -1260,8 +1261,7 @@ cudaError_t ct_launch_zfwd(const ZFwdArgs &a, cudaStream_t s) {
   auto kern = k_zfwd_ct<R, N, V, NOISE>;
   cudaError_t e = set_smem(kern, smem);
   if (e != cudaSuccess) return e;
-  kern<<<persistent_blocks(kern, Pol::THREADS, smem, a.nlines / Pol::L), Pol::THREADS, smem, s>>>(a);
-  return cudaGetLastError();
+  return launch_pass(kern, a.nlines / Pol::L, Pol::THREADS, smem, s, a.overlap, a);
 }
 
 constexpr int kAxisVariants = 3;

@@ -319,6 +319,16 @@ struct LineLayout {
 };
 __host__ __device__ inline int line_ld(int half_len) { return half_len + (half_len >> 4) + 1; }
 
+// Programmatic dependent launch (launch_pass): every kernel that may be launched
+// that way begins with this. The wait ends when the stream's previous kernel is
+// complete and its memory visible; then the next kernel may be brought up, to
+// wait in turn. Nothing is read or written before it. A no-op in a kernel
+// launched the ordinary way.
+__device__ __forceinline__ void pass_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ------------------------------------------------ TMA and mbarrier helpers
 __device__ __forceinline__ uint32_t smem_addr(const void *p) {
   return (uint32_t)__cvta_generic_to_shared(p);

@@ -56,6 +56,7 @@ template <int N, int MODE>
 __global__ void __launch_bounds__(AxisShape<N>::THREADS, AxisShape<N>::MINB)
     k_axis_fx(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap smap0,
               const __grid_constant__ CUtensorMap smap1, const AxisArgs a) {
+  pass_begin();
   using Sh = AxisShape<N>;
   constexpr bool FWD = MODE != kAxisInv, INV = MODE != kAxisFwd;
   constexpr int K = Sh::K, E = Sh::E, P = Sh::P, B = Sh::B, HALF = N / 2, S = ct::nstages(K);
@@ -359,6 +360,7 @@ template <int N, bool NOISE>
 __global__ void __launch_bounds__(ZShape<N>::THREADS,
                                   ZShape<N>::ctas(NOISE ? ZShape<N>::SMEM_COPY : ZShape<N>::SMEM_GEN))
     k_zfwd_fx(const ZFwdArgs a) {
+  pass_begin();
   using Sh = ZShape<N>;
   constexpr int M = Sh::M, K = Sh::K, E = Sh::E, P = Sh::P, L = Sh::L, S = ct::nstages(K);
   constexpr int RF = ct::radix_of(K, 0, false), SPANF = M / RF, NBF = E / RF;
@@ -483,6 +485,7 @@ __global__ void __launch_bounds__(ZShape<N>::THREADS,
 template <int N, bool EXT>
 __global__ void __launch_bounds__(ZShape<N>::THREADS, ZShape<N>::ctas(ZShape<N>::SMEM_COPY + ZShape<N>::Q_BYTES))
     k_zinv_fx(const ZInvArgs a) {
+  pass_begin();
   using Sh = ZShape<N>;
   using R = double;
   constexpr int M = Sh::M, K = Sh::K, E = Sh::E, P = Sh::P, L = Sh::L, S = ct::nstages(K);
@@ -679,8 +682,7 @@ template <int N, int MODE> cudaError_t launch_axis(const AxisArgs &in, cudaStrea
   auto kern = k_axis_fx<N, MODE>;
   if ((e = set_smem(kern, Sh::SMEM)) != cudaSuccess) return e;
   const int64_t tiles = (int64_t)N * a.inner_chunks * (a.nbatch > 0 ? a.nbatch : 1);
-  kern<<<persistent_blocks(kern, Sh::THREADS, Sh::SMEM, tiles), Sh::THREADS, Sh::SMEM, s>>>(map, smap[0], smap[1], a);
-  return cudaGetLastError();
+  return launch_pass(kern, tiles, Sh::THREADS, Sh::SMEM, s, a.overlap, map, smap[0], smap[1], a);
 }
 template <int N, bool NOISE> cudaError_t launch_zfwd(const ZFwdArgs &a, cudaStream_t s) {
   using Sh = ZShape<N>;
@@ -688,8 +690,7 @@ template <int N, bool NOISE> cudaError_t launch_zfwd(const ZFwdArgs &a, cudaStre
   auto kern = k_zfwd_fx<N, NOISE>;
   cudaError_t e = set_smem(kern, smem);
   if (e != cudaSuccess) return e;
-  kern<<<persistent_blocks(kern, Sh::THREADS, smem, a.nlines / Sh::L), Sh::THREADS, smem, s>>>(a);
-  return cudaGetLastError();
+  return launch_pass(kern, a.nlines / Sh::L, Sh::THREADS, smem, s, a.overlap, a);
 }
 template <int N, bool EXT> cudaError_t launch_zinv(const ZInvArgs &a, cudaStream_t s) {
   using Sh = ZShape<N>;
@@ -697,8 +698,7 @@ template <int N, bool EXT> cudaError_t launch_zinv(const ZInvArgs &a, cudaStream
   auto kern = k_zinv_fx<N, EXT>;
   cudaError_t e = set_smem(kern, smem);
   if (e != cudaSuccess) return e;
-  kern<<<persistent_blocks(kern, Sh::THREADS, smem, a.nlines / Sh::L), Sh::THREADS, smem, s>>>(a);
-  return cudaGetLastError();
+  return launch_pass(kern, a.nlines / Sh::L, Sh::THREADS, smem, s, a.overlap, a);
 }
 
 template <int... NS> struct Table {

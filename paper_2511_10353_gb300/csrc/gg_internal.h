@@ -99,6 +99,7 @@ struct AxisArgs {
   // fault test (gg_test_arm_fault): no tile copy is issued, so every CTA's
   // first wait gives up after wait_us and reports GG_ETIMEOUT; 0 normally
   int test_skip_copy;
+  int overlap;            // launch as a programmatic dependent (launch_pass)
   uint32_t wait_us;       // limit of the copy waits in microseconds (0: the default)
 };
 
@@ -118,6 +119,7 @@ struct ZFwdArgs {
   const uint64_t *seeds;  // batched form: device array, one seed per realization (else seed)
   int64_t lines_per_real; // lines of one realization (<= 0: nlines)
   int *err;               // device error word (caller noise: a copy wait gave up)
+  int overlap;            // launch as a programmatic dependent (launch_pass)
 };
 
 // One axis of a separable spectral filter on real lines along z (F32 sizes with
@@ -131,6 +133,7 @@ struct ZFilterArgs {
   const void *tw_half;
   const void *tw_full;
   int *err;
+  int overlap;            // launch as a programmatic dependent (launch_pass)
 };
 
 // Inverse z pass (c2r) with the Zel'dovich epilogue (Eq. 3) or a plain real
@@ -166,6 +169,7 @@ struct ZInvArgs {
   // the transform's output before the epilogue; nullptr: none
   const void *large;
   int n_low;
+  int overlap;            // launch as a programmatic dependent (launch_pass)
   int large_rows;         // coarse lines staged per tile (set by the launcher; 0: none)
   // Sec. 2.2 particle options: shift added to q for pos (periodic shift, and
   // the dark-matter offset of gas pairs); pos2: a second position output
@@ -249,8 +253,8 @@ template <typename R> cudaError_t launch_axis(const AxisArgs &a, cudaStream_t s)
 template <typename R> cudaError_t launch_zinv(const ZInvArgs &a, cudaStream_t s);
 template <typename R> int max_block_threads_z(int kind, int e);  // kind 0: z forward, 2: z inverse
 template <typename R> int max_block_threads_axis(int e);
-// Size-specialised kernels (gg_ct_f32.cu / gg_ct_f64.cu) for the grid sizes of
-// the named workloads; spec_has tells whether N has them.
+// Size-specialised kernels: FP32 in gg_ct_f32.cu and gg_ct_more_f32.cu, FP64 in
+// gg_fx_axis.cu and gg_fx_z.cu; spec_has tells whether N has them.
 template <typename R> bool spec_has(int n);
 template <typename R> bool spec_tuned(int n);  // has tile variants (gg_autotune)
 template <typename R> bool spec_three_ctas(int n);  // strided variant 2: three CTAs an SM

@@ -48,6 +48,7 @@ __global__ void k_noise(NoiseArgs a) {
 // k < N/2 (the real-input DFT).
 template <typename R, int E>
 __global__ void k_zfwd(const ZFwdArgs a) {
+  pass_begin();
   using C = Cx<R>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   C *buf = reinterpret_cast<C *>(smem_raw);
@@ -129,6 +130,7 @@ __device__ __forceinline__ Cx<R> apply_mul(int kind, Cx<R> v, int n, int N) {
 template <typename R, int E>
 __global__ void __launch_bounds__(E >= 24 ? 256 : 512, 1)
     k_axis(const __grid_constant__ CUtensorMap map, const AxisArgs a) {
+  pass_begin();
   using C = Cx<R>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   uint64_t *bars = reinterpret_cast<uint64_t *>(smem_raw);
@@ -311,6 +313,7 @@ __global__ void __launch_bounds__(E >= 24 ? 256 : 512, 1)
 // mod L, vel = vfac psi; or the plain real field when pos and vel are null.
 template <typename R, int E>
 __global__ void k_zinv(const ZInvArgs a) {
+  pass_begin();
   using C = Cx<R>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   C *buf = reinterpret_cast<C *>(smem_raw);
@@ -438,9 +441,8 @@ cudaError_t launch_zfwd(const ZFwdArgs &a, cudaStream_t s) {
     auto kern = k_zfwd<R, EE>;
     cudaError_t e = set_smem(kern, smem);
     if (e != cudaSuccess) return e;
-    kern<<<blocks, threads, smem, s>>>(a);
+    return launch_pass<false>(kern, blocks, (int)threads, smem, s, a.overlap, a);
   });
-  return cudaGetLastError();
 }
 
 template <typename R>
@@ -456,9 +458,8 @@ cudaError_t launch_axis(const AxisArgs &a, cudaStream_t s) {
   GG_DISPATCH_E(a.e, {
     auto kern = k_axis<R, EE>;
     if ((e = set_smem(kern, smem)) != cudaSuccess) return e;
-    kern<<<persistent_blocks(kern, threads, smem, tiles), threads, smem, s>>>(map, a);
+    return launch_pass(kern, tiles, (int)threads, smem, s, a.overlap, map, a);
   });
-  return cudaGetLastError();
 }
 
 template <typename R>
@@ -471,9 +472,8 @@ cudaError_t launch_zinv(const ZInvArgs &a, cudaStream_t s) {
     auto kern = k_zinv<R, EE>;
     cudaError_t e = set_smem(kern, smem);
     if (e != cudaSuccess) return e;
-    kern<<<blocks, threads, smem, s>>>(a);
+    return launch_pass<false>(kern, blocks, (int)threads, smem, s, a.overlap, a);
   });
-  return cudaGetLastError();
 }
 
 // Largest block each kernel can launch with (registers bound it), so the host
