@@ -193,13 +193,14 @@ gg_status gg_set_profiling(gg_plan_t *plan, int enable);
 gg_status gg_profile_read(gg_plan_t *plan, int reset, int *count, const char **names, double *ms,
                           int64_t *launches, double *bytes);
 
-/* Autotuner of the transform tiles (grid sizes with size-specialised kernels:
- * N = 64, 128, 192, 256, 384, 512, 1536 in FP32; 64, 512, 1536 in FP64; the
- * other specialised sizes have one tile shape).
+/* Autotuner of the transform tiles (grid sizes with several tile shapes:
+ * N = 64, 128, 192, 256, 384, 512, 1536 in FP32; a new plan starts with the
+ * shapes measured best at its size).
  * Runs the whole path `reps` times per tile variant on the plan's own buffers
  * (allocating the component workspaces and one scratch grid for the call),
  * times each pass with CUDA events and keeps the fastest variant per pass for
- * later calls. Synchronous. Other sizes: returns GG_OK and changes nothing.
+ * later calls. Synchronous. Other sizes, and FP64, have one shape: returns
+ * GG_OK and changes nothing.
  * Results do not depend on the variant (same arithmetic, different tiling). */
 gg_status gg_autotune(gg_plan_t *plan, int reps);
 

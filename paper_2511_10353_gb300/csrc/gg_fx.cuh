@@ -5,8 +5,8 @@
 // instructions a point, 14 SM cycles, however it is scheduled, and the FP64
 // kernels ran at 84% of that bound. The same transform on 64-bit integers takes
 // about 120 integer instructions a point, two to three cycles. 512^3 noise ->
-// pos + vel 59.1 -> 12.3 ms (z forward 12.9 -> 2.32, y 3.38 -> 0.86, x 11.1 -> 2.95,
-// y inverses 11.0 -> 2.54, z inverses 20.7 -> 3.61), bound by the latency of the
+// pos + vel 59.1 -> 12.8 ms (z forward 12.9 -> 2.39, y 3.38 -> 0.90, x 11.1 -> 3.09,
+// y inverses 11.0 -> 2.67, z inverses 20.7 -> 3.68), bound by the latency of the
 // integer chains at 16 to 20 warps an SM.
 //
 // Each transform of N points (a column of a tile, a line) gets one power of two
