@@ -583,13 +583,12 @@ constexpr int kPersistV = 4;
 
 // Sizes with several tile variants for the autotuner (the named workloads'
 // and their neighbours); every other size has the one shape of variant 0.
-template <typename R> __host__ __device__ constexpr bool ct_tuned(int n) {
-  if (sizeof(R) == 8) return n == 64 || n == 512 || n == 1536;
+__host__ __device__ constexpr bool ct_tuned(int n) {
   return n == 64 || n == 128 || n == 192 || n == 256 || n == 384 || n == 512 || n == 1536;
 }
 
 template <typename R, int N, int V> struct AxisPolicy {
-  static constexpr bool TUNED = ct_tuned<R>(N);
+  static constexpr bool TUNED = ct_tuned(N);
   static constexpr int CB = 2 * (int)sizeof(R);
   static constexpr bool BIG = is_big(skey<R>(N));
   static constexpr int E0 = elems(skey<R>(N));

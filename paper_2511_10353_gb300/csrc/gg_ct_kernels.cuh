@@ -1272,7 +1272,7 @@ template <typename R, int... NS> struct CtTable {
   static bool has(int n) { return ((n == NS) || ...); }
   static bool three(int n) { return ((n == NS && ct::AxisPolicy<R, NS, 2>::THREE) || ...); }
   template <int N> static int cols_n(int v) {
-    if constexpr (!ct::ct_tuned<R>(N)) return ct::AxisPolicy<R, N, 0>::B;
+    if constexpr (!ct::ct_tuned(N)) return ct::AxisPolicy<R, N, 0>::B;
     else return v == 1 ? ct::AxisPolicy<R, N, 1>::B : (v == 2 ? ct::AxisPolicy<R, N, 2>::B : ct::AxisPolicy<R, N, 0>::B);
   }
   static int cols(int n, int v) {
@@ -1302,7 +1302,7 @@ template <typename R, int... NS> struct CtTable {
       if (a.interp) return ct_launch_axis<R, N, V, kAxisFwdInv, true, kFiltInterp>(a, s);
       return ct_launch_axis<R, N, V, kAxisFwdInv, true>(a, s);
     }
-    if constexpr (ct::ct_tuned<R>(N)) {
+    if constexpr (ct::ct_tuned(N)) {
       if (a.variant == 1) return axis_v<N, 1>(a, s);
       if (a.variant == 2) return axis_v<N, 2>(a, s);
     }
@@ -1357,7 +1357,7 @@ template <typename R, int... NS> struct CtTable {
       return a.comp == 2 ? ct_launch_zinv<R, N, 0, true, kZPosVelZ>(a, s)
                          : ct_launch_zinv<R, N, 0, true, kZPosVel>(a, s);
     }
-    if constexpr (ct::ct_tuned<R>(N)) {
+    if constexpr (ct::ct_tuned(N)) {
       if (a.variant == 1) return zinv_v<N, 1>(a, s);
       if (a.variant == 2) return zinv_v<N, 2>(a, s);
       if (a.variant == 3) return zinv_v<N, 3>(a, s);
@@ -1368,7 +1368,7 @@ template <typename R, int... NS> struct CtTable {
     return a.noise ? ct_launch_zfwd<R, N, V, true>(a, s) : ct_launch_zfwd<R, N, V, false>(a, s);
   }
   template <int N> static cudaError_t zfwd_n(const ZFwdArgs &a, cudaStream_t s) {
-    if constexpr (ct::ct_tuned<R>(N)) {
+    if constexpr (ct::ct_tuned(N)) {
       if (a.variant == 1) return zfwd_v<N, 1>(a, s);
       if (a.variant == 2) return zfwd_v<N, 2>(a, s);
       if (a.variant == 3) return zfwd_v<N, 3>(a, s);
