@@ -110,6 +110,9 @@ struct gg_plan {
   // set for the duration of a call: the run-time kernels also where N has
   // specialised ones (run_power_spectrum)
   bool runtime_kernels = false;
+  // the strided forward passes take the general radices (8, 4, 2, 3) where a
+  // codelet has a schedule of its own in their place (N = 384; the power spectrum)
+  int general_radices = 0;
   double *diag = nullptr;  // device sums of the diagnostics, grown on use
   size_t diag_words = 0;
 };
@@ -488,6 +491,7 @@ gg::AxisArgs axis_args(gg_plan_t *plan, int axis, const void *src) {
   c.e = plan->col_e;
   c.rows_box = plan->col_rows_box;
   c.overlap = plan->overlap;
+  c.general_radices = plan->general_radices;
   c.err = plan->err;
   return c;
 }
@@ -1261,8 +1265,10 @@ gg_status run_power_spectrum(gg_plan_t *plan, const void *field, int nbins, doub
   if (st != GG_OK) return st;
   // P(k) is returned in FP64, where another rounding of the FP32 transforms shows
   // (1e-8): the FP32 sizes whose specialised kernels have one tile shape keep
-  // the run-time kernels' arithmetic here
+  // the run-time kernels' arithmetic here, and 384 the 8 x 8 x 2 x 3 of the
+  // other passes' 8 x 8 x 6
   plan->runtime_kernels = sizeof(R) == 4 && !gg::spec_tuned<R>(n);
+  plan->general_radices = 1;
   st = forward_zy<R>(plan, 0, field);
   if (st == GG_OK) {
     gg::AxisArgs x = axis_args<R>(plan, 0, plan->work);
@@ -1275,6 +1281,7 @@ gg_status run_power_spectrum(gg_plan_t *plan, const void *field, int nbins, doub
     st = launch_axis_timed<R>(plan, x, kXFused, "x forward pass");
   }
   plan->runtime_kernels = false;
+  plan->general_radices = 0;
   if (st != GG_OK) return st;
   double *sums = plan->diag;
   cudaError_t e = cudaSuccess;

@@ -21,6 +21,9 @@ struct Line512 {
 };
 struct Line384 {
   float v;
+  Line384() = default;
+  __host__ __device__ constexpr Line384(float x) : v(x) {}
+  __host__ __device__ constexpr operator float() const { return v; }
 };
 template <> struct CxOf<Line512> { using T = float2; };
 template <> struct CxOf<Line384> { using T = float2; };

@@ -272,7 +272,7 @@ __device__ __forceinline__ bool axis_body(const CUtensorMap &map, const AxisArgs
 #pragma unroll
         for (int r = 0; r < RH; ++r)
           X[b * RH + r] = cmul(X[b * RH + r], ldg_c(fac + p + P * b + r * SPAN));
-    } else if (pre) {
+    } else if constexpr (FILT != kFiltNone) if (pre) {
 #pragma unroll
       for (int b = 0; b < NB; ++b)
 #pragma unroll
@@ -1302,6 +1302,9 @@ template <typename R, int... NS> struct CtTable {
       if (a.interp) return ct_launch_axis<R, N, V, kAxisFwdInv, true, kFiltInterp>(a, s);
       return ct_launch_axis<R, N, V, kAxisFwdInv, true>(a, s);
     }
+    if constexpr (N == 384 && std::is_same<R, float>::value)
+      if (a.general_radices && a.fwd && !a.inv && !a.pre)
+        return ct_launch_axis<Line384, N, 0, kAxisFwd, false, kFiltNone>(a, s);
     if constexpr (ct::ct_tuned(N)) {
       if (a.variant == 1) return axis_v<N, 1>(a, s);
       if (a.variant == 2) return axis_v<N, 2>(a, s);

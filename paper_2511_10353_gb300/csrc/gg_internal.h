@@ -100,6 +100,7 @@ struct AxisArgs {
   // first wait gives up after wait_us and reports GG_ETIMEOUT; 0 normally
   int test_skip_copy;
   int overlap;            // launch as a programmatic dependent (launch_pass)
+  int general_radices;    // forward only: the general schedule's rounding (Line384)
   uint32_t wait_us;       // limit of the copy waits in microseconds (0: the default)
 };
 
