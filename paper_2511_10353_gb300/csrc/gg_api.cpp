@@ -262,12 +262,42 @@ std::vector<int32_t> fixed_table(int len) {
   return t;
 }
 
+// Pageable host memory to the device, complete on return: cudaMemcpy may return
+// with the last part still on its way, which a launch on a stream that does not
+// wait for the legacy one could overtake.
+cudaError_t copy_to_device(void *dst, const void *src, size_t bytes) {
+  const cudaError_t e = cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice);
+  return e == cudaSuccess ? cudaStreamSynchronize(cudaStreamLegacy) : e;
+}
+
 template <typename R>
 gg_status upload(gg_plan_t *plan, void **dst, const std::vector<R> &v) {
   cudaError_t e = cudaMalloc(dst, v.size() * sizeof(R));
   if (e != cudaSuccess) return fail(plan, GG_ENOMEM, "cudaMalloc (tables) failed");
-  e = cudaMemcpy(*dst, v.data(), v.size() * sizeof(R), cudaMemcpyHostToDevice);
+  e = copy_to_device(*dst, v.data(), v.size() * sizeof(R));
   if (e != cudaSuccess) return cuda_fail(plan, e, "cudaMemcpy (tables)");
+  return GG_OK;
+}
+
+// New values into plan->tab.smooth. The passes of the radius before may still be
+// queued on the plan's stream (often one that does not wait for the legacy
+// stream of cudaMemcpy): they are waited for first. A capture in progress has
+// nothing queued to wait for.
+template <typename R>
+gg_status replace_smooth(gg_plan_t *plan, double radius, const std::vector<R> &v) {
+  const size_t bytes = v.size() * sizeof(R);
+  cudaError_t e;
+  if (!plan->tab.smooth && (e = cudaMalloc(&plan->tab.smooth, bytes)) != cudaSuccess) {
+    plan->tab.smooth = nullptr;
+    return fail(plan, GG_ENOMEM, "cudaMalloc of the smoothing table failed");
+  }
+  plan->tab.smooth_radius = -1.0;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  e = cudaStreamIsCapturing(plan->stream, &cap);
+  if (e == cudaSuccess && cap == cudaStreamCaptureStatusNone) e = cudaStreamSynchronize(plan->stream);
+  if (e == cudaSuccess) e = copy_to_device(plan->tab.smooth, v.data(), bytes);
+  if (e != cudaSuccess) return cuda_fail(plan, e, "smoothing table upload");
+  plan->tab.smooth_radius = radius;
   return GG_OK;
 }
 
@@ -1169,14 +1199,8 @@ gg_status run_smooth_separable(gg_plan_t *plan, double radius, const void *in, v
       const double m = (double)(i < n / 2 ? i : i - n);
       if (i != n / 2) t[2 * i] = (float)(std::exp(-0.5 * kf * kf * m * m * radius * radius) / (double)n);
     }
-    cudaError_t e;
-    if (!plan->tab.smooth && (e = cudaMalloc(&plan->tab.smooth, t.size() * sizeof(float))) != cudaSuccess)
-      return fail(plan, GG_ENOMEM, "cudaMalloc of the smoothing table failed");
-    plan->tab.smooth_radius = -1.0;
-    if ((e = cudaMemcpy(plan->tab.smooth, t.data(), t.size() * sizeof(float), cudaMemcpyHostToDevice)) !=
-        cudaSuccess)
-      return cuda_fail(plan, e, "smoothing table upload");
-    plan->tab.smooth_radius = radius;
+    const gg_status st = replace_smooth(plan, radius, t);
+    if (st != GG_OK) return st;
   }
   return run_separable(plan, plan->tab.smooth, in, out);
 }
@@ -1191,13 +1215,8 @@ gg_status run_smooth(gg_plan_t *plan, double radius, const void *in, void *out) 
     const double kf = 2.0 * kPi / plan->p.box;
     const double n3 = (double)n * n * n;
     for (size_t i = 0; i < cnt; ++i) t[i] = (R)(std::exp(-0.5 * kf * kf * (double)i * radius * radius) / n3);
-    cudaError_t e;
-    if (!plan->tab.smooth && (e = cudaMalloc(&plan->tab.smooth, cnt * sizeof(R))) != cudaSuccess)
-      return fail(plan, GG_ENOMEM, "cudaMalloc of the smoothing table failed");
-    if ((e = cudaMemcpy(plan->tab.smooth, t.data(), cnt * sizeof(R), cudaMemcpyHostToDevice)) !=
-        cudaSuccess)
-      return cuda_fail(plan, e, "smoothing table upload");
-    plan->tab.smooth_radius = radius;
+    const gg_status st = replace_smooth(plan, radius, t);
+    if (st != GG_OK) return st;
   }
   return run_density<R>(plan, 0, in, out, plan->tab.smooth);
 }
