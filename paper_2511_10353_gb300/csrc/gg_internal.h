@@ -329,6 +329,13 @@ cudaError_t launch_persist(PersistPlan p, cudaStream_t s, int *launched_blocks);
 // device: asked once for each (a few hundred entries at most; any thread).
 int resident_blocks(const void *kernel, int threads, size_t smem);
 
+// Lets a kernel be launched with `bytes` of dynamic shared memory on the current
+// device. The limit belongs to the kernel, not to a launch, and the bytes of one
+// kernel vary with the call (grid size, coarse grid, bins): it is only ever
+// raised, so that plans on several host threads cannot take it from under each
+// other between this call and the launch.
+cudaError_t raise_smem(const void *kernel, size_t bytes);
+
 // Message returned by gg_last_error(NULL) on this host thread.
 void set_thread_error(const char *msg);
 cudaError_t launch_noise_bits(uint64_t seed, int64_t first, int64_t count, uint32_t *out,

@@ -3,6 +3,7 @@
 #include <map>
 #include <mutex>
 #include <tuple>
+#include <utility>
 
 #include "gg_device.cuh"
 
@@ -43,6 +44,20 @@ int resident_blocks(const void *kernel, int threads, size_t smem) {
   std::lock_guard<std::mutex> lock(mu);
   known[key] = sms * per;
   return sms * per;
+}
+
+cudaError_t raise_smem(const void *kernel, size_t bytes) {
+  if (bytes <= 48 * 1024) return cudaSuccess;
+  static std::mutex mu;
+  static std::map<std::pair<const void *, int>, size_t> limits;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  std::lock_guard<std::mutex> lock(mu);  // around the call too: limits arrive in rising order
+  size_t &limit = limits[{kernel, dev}];
+  const size_t want = bytes > limit ? bytes : limit;
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)want);
+  if (e == cudaSuccess) limit = want;
+  return e;
 }
 
 size_t zpass_smem_bytes(int half_len, int lines, size_t complex_bytes) {

@@ -12,10 +12,8 @@
 
 namespace gg {
 
-template <typename K>
-static cudaError_t set_smem(K kernel, size_t bytes) {
-  if (bytes <= 48 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+template <typename K> static cudaError_t set_smem(K kernel, size_t bytes) {
+  return raise_smem(reinterpret_cast<const void *>(kernel), bytes);
 }
 
 using EncodeTiledFn = PFN_cuTensorMapEncodeTiled_v12000;

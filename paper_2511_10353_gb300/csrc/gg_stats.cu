@@ -305,10 +305,8 @@ int grid_for(int64_t work, int per_sm) {
 template <typename K> cudaError_t shell_launch(K kern, const ShellArgs &a, int copies, size_t per_copy, int blocks,
                                                cudaStream_t s) {
   const size_t smem = per_copy * copies;
-  if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = raise_smem(reinterpret_cast<const void *>(kern), smem);
+  if (e != cudaSuccess) return e;
   kern<<<blocks, 256, smem, s>>>(a, copies);
   return cudaGetLastError();
 }

@@ -1,6 +1,8 @@
-"""Calls that follow each other on a side stream without a synchronisation give
-the results of lone calls.
+"""Calls that follow each other on a side stream without a synchronisation, and
+distinct plans on several host threads: results equal those of lone calls.
 """
+import threading
+
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -42,3 +44,29 @@ def test_smoothing_radii_back_to_back(gg, n, prec):
         for q in range(reps):
             assert torch.equal(got[i * reps + q], want[i]), (radii[i], q)
     plan.close()
+
+
+def test_merges_on_two_threads(gg):
+    """Coarse grids of different sizes need different shared memory in one kernel."""
+    n, box, runs = 512, 500.0, 150
+    errors = []
+
+    def work(nl, seed):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                plan = gg.Plan(n, box, BBKS, 20.0, "f32")
+                large = [torch.full((nl, nl, nl), 0.01, device="cuda") for _ in range(3)]
+                out = {"psi": [plan.empty() for _ in range(3)], "pos": [None] * 3, "vel": [None] * 3}
+                for _ in range(runs):
+                    plan.zeldovich_merge(large, 2 * box / nl, seed=seed, out=out)
+                plan.sync()
+                plan.close()
+        except Exception as e:  # reported by the test's thread
+            errors.append((nl, repr(e)))
+
+    threads = [threading.Thread(target=work, args=(nl, i)) for i, nl in enumerate((256, 128))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
