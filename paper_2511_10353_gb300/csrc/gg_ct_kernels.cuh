@@ -858,7 +858,7 @@ __device__ __forceinline__ bool zinv_body(const ZInvArgs &a, int64_t t0, int64_t
           const R c1 = w0 * r0[tap.z + 1] + w1 * r1[tap.z + 1];
           const R c2 = w0 * r0[tap.z + 2] + w1 * r1[tap.z + 2];
           z.x += tap.a0 * c0 + tap.a1 * c1;
-          z.y += tap.b0 * c0 + tap.b1 * c1 + tap.b2 * c2;
+          z.y += tap.b0 * (tap.step ? c1 : c0) + tap.b1 * (tap.step ? c2 : c1);
         });
       } else if (large) {
         each([&](int n, C &z) {

@@ -226,22 +226,23 @@ __device__ __forceinline__ void cic_pair(const R *__restrict__ g, int nl, int nh
   a1 = step ? ((R)1 - t1) * c1 + t1 * c2 : ((R)1 - t1) * c0 + t1 * c1;
 }
 
-// The z part of cic_pair for cells 2n and 2n + 1: their weights of the three
-// coarse cells z, z + 1, z + 2 (the first cell uses two).
+// The z part of cic_pair for cells 2n and 2n + 1: their weights of two coarse
+// cells each, z and z + 1, or (the second cell, where step is set) z + 1 and
+// z + 2. A cell's value is formed from its own two only: a third at weight zero
+// would spread an infinity or a NaN there.
 template <typename R> struct MergeTap {
-  R a0, a1, b0, b1, b2;
-  int z;
+  R a0, a1, b0, b1;
+  int z, step;
 };
 template <typename R> __device__ __forceinline__ MergeTap<R> merge_tap(int nl, int nh, int n) {
   const int den = 2 * nh;
   const int num0 = (4 * n + 1) * nl - nh;
   const int q = num0 >= 0 ? num0 / den : -((den - 1 - num0) / den);  // floor, >= -1
   const int r0 = num0 - q * den;
-  const bool step = r0 + 2 * nl >= den;  // cell 2n + 1 starts one coarse cell later
-  const int r1 = r0 + 2 * nl - (step ? den : 0);
+  const int step = r0 + 2 * nl >= den ? 1 : 0;  // cell 2n + 1 starts one coarse cell later
+  const int r1 = r0 + 2 * nl - step * den;
   const R t0 = (R)r0 / (R)den, t1 = (R)r1 / (R)den;
-  return MergeTap<R>{(R)1 - t0, t0, step ? (R)0 : (R)1 - t1, step ? (R)1 - t1 : t1, step ? t1 : (R)0,
-                     q < 0 ? q + nl : q};
+  return MergeTap<R>{(R)1 - t0, t0, (R)1 - t1, t1, q < 0 ? q + nl : q, step};
 }
 
 // ------------------------------------------------------------------ butterflies
