@@ -10,15 +10,25 @@
 // integer chains at 16 to 20 warps an SM.
 //
 // Each transform of N points (a column of a tile, a line) gets one power of two
-// as its scale, from the sum of |re| + |im| of its inputs (col_scale): the
-// largest one for which that sum stays below 2^62. Every intermediate and
-// output of the transform is bounded by the same sum (all twiddles have modulus
-// one), so nothing overflows: 64-bit signed values hold twice that. With s the
-// sum and L2 the root of the sum of squares of the inputs (s <= sqrt(2 N) L2),
-// rounding the inputs to units of s 2^-62 changes the outputs by at most
-// 0.41 sqrt(2 N) sqrt(N) 2^-62 L2 against outputs of rms L2: below 2^-53 for
-// every input up to N = 512, less than the FP64 transform's own rounding (nine
-// levels of 2^-53 each and its twiddles). Products by twiddles keep 62 bits.
+// as its scale, from the sum A of the moduli of its inputs, estimated from above by
+// the sum of |re| + |im|, above N = 768 more closely (modulus): the largest one for
+// which that stays below 2^62.5. Every intermediate and output of the transform is
+// bounded by A (all twiddles have modulus one), and the sums re + im that products
+// by (1 + i) / sqrt(2) take by sqrt(2) A, so nothing reaches 2^63. (z forward, whose
+// last step adds two outputs, and the i m outputs of the strided passes: 2^62.)
+//
+// Rounding the inputs to their unit u changes each output by 0.41 sqrt(N) u rms.
+// The unit is A 2^-62.5 to A 2^-61.5 and A <= sqrt(N) L2 (L2: root of the sum of
+// squares of the inputs, the rms of the outputs), so a flat spectrum or white
+// noise is off by up to 0.41 N 2^-61.5 of its rms, a steep one by less. Products by
+// twiddles keep 62 bits; those of the first stages add a third. Emulated for a
+// strided column of white noise, rms over the position of the power of two: 1.1e-16
+// at N = 1024, 1.8e-16 at 1536 (an FP64 transform there: 2.5e-16, 2.7e-16).
+// Six transforms forward and back on white noise, against the identity, fixed
+// point and FP64 transforms:
+//   N             64    256   384   512   768   1024  1536
+//   fixed point   1.5   1.6   2.8   2.2   3.4   3.0   4.4   e-16 relative L2 (largest: 4.7)
+//   FP64          4.3   5.4   5.8   5.7   6.2   6.2   6.6
 // Measured against 113-bit arithmetic, the density chain of six transforms is
 // off by 1.2e-16 to 2.7e-16 relative L2 (white, steep, spike and single-mode
 // fields of 32^3 to 128^3; the FP64 transforms: 3.0e-16 to 5.2e-16).
@@ -35,6 +45,7 @@ template <> struct CxOf<long long> { using T = Fx; };
 
 namespace fx {
 
+constexpr float kRootHalf = 0.70710684f;                // sqrt(1/2), from above
 constexpr long long kSqrtHalf = 3260954456333195553ll;  // sqrt(1/2) 2^62
 constexpr long long kSin60 = 3993837246235628775ll;     // sqrt(3)/2 2^62
 
@@ -81,7 +92,8 @@ namespace fx {
 
 // ------------------------------------------------------------ scale and conversion
 __device__ __forceinline__ uint32_t mag_hi(double v) { return (uint32_t)__double2hiint(v) & 0x7fffffffu; }
-// |value| / 2^(e - 1023) from its high word (20 mantissa bits; 0 below 2^-126)
+// |value| / 2^(e - 1023) from its high word (20 mantissa bits; 0 below 2^-126; for
+// values up to 2^128 above 2^(e - 1023))
 __device__ __forceinline__ float rel(uint32_t h, int e) {
   const int v = (int)h - ((e - 127) << 20);
   return __int_as_float((v > 0 ? v : 0) << 3);
@@ -92,16 +104,18 @@ __device__ __forceinline__ float pow2(int e) {  // 2^e, 0 below -126, for e <= 0
 
 // Scale of a transform: values are integers in units of 2^-s; k: see to_fixed.
 struct Scale {
-  int k, s;
+  int k, s, e;
   bool bad;  // an infinity or a NaN among the inputs
 };
-// e: largest biased exponent; sum: sum of |re| + |im| in units of 2^(e - 1023)
+// e: largest biased exponent; sum: the transform's bound in units of 2^(e - 1023)
 __device__ __forceinline__ Scale scale_of(int e, float sum) {
   Scale c;
-  // sum 1.0001 covers the truncated mantissas and the FP32 rounding
-  const int es = (int)(__float_as_uint(sum * 1.0001f + 1e-30f) >> 23) - 127;
+  // sum 1.0001 covers the truncated mantissas and the FP32 rounding; es below 0
+  // would take a lone value out of to_fixed's range
+  const int es = (int)(__float_as_uint(fmaxf(sum * 1.0001f, 1.0f)) >> 23) - 127;
   c.s = 1084 - e - es;   // the sum times 2^s is below 2^62
   c.k = 1075 - c.s;
+  c.e = e;
   c.bad = e == 2047;
   return c;
 }
@@ -132,10 +146,10 @@ __device__ __forceinline__ long long to_fixed(double v, const Scale &sc, const W
   const uint32_t mh = (hi & 0xfffffu) | 0x100000u;
   const unsigned long long p = (unsigned long long)lo * w.m;
   const unsigned long long m = p + ((unsigned long long)(mh * w.m) << 32);
-  // m >= 2^62 and the result is below 2^62: r >= 1. Rounded to nearest: cutting
-  // off would shrink every transform by up to 2^-53.
-  int r = sc.k + w.c - e - 1;
-  r = r < 63 ? r : 63;
+  // m >= 2^62 and the result is below 2^62: r >= 0, except for a value dropped by
+  // its weight (m = 0), whose r may be anything. Rounded to nearest: cutting off
+  // would shrink every transform by up to 2^-53.
+  const uint32_t r = min((uint32_t)(sc.k + w.c - e - 1), 63u);
   unsigned long long f = ((m >> r) + 1) >> 1;
   if (e == 0) f = 0;  // zeros and subnormals
   const long long g = (long long)f;
@@ -199,7 +213,15 @@ __device__ __forceinline__ int max_exp(int e, double2 v) {
   const int x = (int)((a > b ? a : b) >> 20);
   return e > x ? e : x;
 }
-__device__ __forceinline__ float rel2(double2 v, int e) { return rel(mag_hi(v.x), e) + rel(mag_hi(v.y), e); }
+// the grids that need every bit of the block scale (see the head of the file)
+__host__ __device__ constexpr bool fine(int n) { return n > 768; }
+// modulus of v / 2^(e - 1023), from above: max + (sqrt(2) - 1) min, within 1.083 of it,
+// where a quarter bit counts; else |re| + |im| (two instructions a value less: 1% of
+// a run at 64^3 and 512^3)
+template <int N> __device__ __forceinline__ float modulus(double2 v, int e) {
+  const float a = rel(mag_hi(v.x), e), b = rel(mag_hi(v.y), e);
+  return fine(N) ? fmaf(fminf(a, b), 0.41421357f, fmaxf(a, b)) : a + b;
+}
 
 }  // namespace fx
 }  // namespace gg

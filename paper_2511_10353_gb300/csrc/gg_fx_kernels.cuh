@@ -204,8 +204,8 @@ __global__ void __launch_bounds__(AxisShape<N>::THREADS, AxisShape<N>::MINB)
             [&](int e) {
               float s = 0.0f;
 #pragma unroll
-              for (int i = 0; i < E; ++i) s += rel2(d[i], e);
-              return s;
+              for (int i = 0; i < E; ++i) s += modulus<N>(d[i], e);
+              return kRootHalf * s;
             });  // its barrier: every thread has read the tile
         const Weight one = weight_one();
 #pragma unroll
@@ -276,7 +276,11 @@ __global__ void __launch_bounds__(AxisShape<N>::THREADS, AxisShape<N>::MINB)
           [&](int e) {
             float s = 0.0f;
 #pragma unroll
-            for (int i = 0; i < E; ++i) s += rel2(X[i], e) * (im ? fabsf((float)freq(i)) : 1.0f);
+            for (int i = 0; i < E; ++i) {
+              const float x = modulus<N>(X[i], e);
+              // i m: without the half bit, so that a lone weighted value stays in to_fixed's range
+              s += im ? (freq(i) == 0 ? 0.0f : x * fabsf((float)freq(i))) : kRootHalf * x;
+            }
             return s;
           });  // its barrier: every thread has read the work tile
       Fx v[E];
@@ -436,8 +440,8 @@ __global__ void __launch_bounds__(ZShape<N>::THREADS,
           [&](int e) {
             float s = 0.0f;
 #pragma unroll
-            for (int i = 0; i < E; ++i) s += rel2(d[i], e);
-            return s;
+            for (int i = 0; i < E; ++i) s += modulus<N>(d[i], e);
+            return s;  // the pairs' sums Z_k + conj Z_{M-k} are twice as large
           });  // its barrier: every thread has read its values
       if constexpr (NOISE) {
         if (tid == 0 && t + gridDim.x < ntiles) {
@@ -480,8 +484,19 @@ __global__ void __launch_bounds__(ZShape<N>::THREADS,
   }
 }
 
-// The inverse z pass and the Eq. 3 epilogue (see zinv_body). The pairs of the
-// c2r pre-processing add up to four times their inputs' sum: two bits less.
+// The inverse z pass and the Eq. 3 epilogue (see zinv_body). A pair of the c2r
+// pre-processing, Z_k = S + T and Z_{M-k} = conj(S - T), has |Z_k|^2 + |Z_{M-k}|^2 =
+// 4 (|X_k|^2 + |X_{M-k}|^2): the line's sum of moduli grows by at most 2 sqrt(2),
+// and each value fits far below it. Lines above 384 (N > 768) form the pairs in a
+// finer unit (2^-g of the transform's, g from the line: six bits on a flat spectrum)
+// and round them once, so that the transform's inputs carry one rounding at its
+// unit instead of those of four inputs, which alone came to 5e-16 at N = 1536. At N =
+// 512 (2.9e-16 for six transforms without it) it would cost 1.5% of the run.
+__host__ __device__ constexpr int im_bits(int m) {  // frequencies below m are below 2^im_bits
+  int b = 0;
+  while ((1 << b) < m) ++b;
+  return b;
+}
 template <int N, bool EXT>
 __global__ void __launch_bounds__(ZShape<N>::THREADS, ZShape<N>::ctas(ZShape<N>::SMEM_COPY + ZShape<N>::Q_BYTES))
     k_zinv_fx(const ZInvArgs a) {
@@ -549,40 +564,49 @@ __global__ void __launch_bounds__(ZShape<N>::THREADS, ZShape<N>::ctas(ZShape<N>:
 #pragma unroll
             for (int i = 0; i < E / 2; ++i) {
               const int k = p + P * i;
-              s += rel2(xk[i], e) * (im ? (float)k : 1.0f) +
-                   rel2(xm[i], e) * (im ? (float)(k ? M - k : M / 2) : 1.0f);
+              const float x = modulus<N>(xk[i], e), y = modulus<N>(xm[i], e);
+              s += im ? (k ? x * (float)k : 0.0f) + y * (float)(k ? M - k : M / 2) : x + y;
             }
-            return 4.0f * s;
+            return 2.0f * s;  // sum of |Z| below 2^62.5
           });  // its barrier: the dense tile has been read
       if (tid == 0 && t + gridDim.x < ntiles) {
         fence_proxy_async_smem();
         issue(t + gridDim.x);
       }
+      Scale su = sc;
+      int g = 0;
+      if constexpr (fine(N)) {  // weighted inputs stay below 2^60 in the finer unit
+        const int room = 1082 - sc.s - sc.e - (im ? im_bits(M) : 0);
+        g = room < 0 ? 0 : (room < 6 ? room : 6);
+        su.k -= g;
+      }
+      const I half = (1ll << g) >> 1;
+      auto put = [&](int n, Fx v) { st(n, Fx{(v.x + half) >> g, (v.y + half) >> g}); };
 #pragma unroll
       for (int i = 0; i < E / 2; ++i) {
         const int k = p + P * i, km = k ? M - k : M / 2;
         Fx u, w;
         if (im) {  // i m_z on both members
           Weight wk = weight_int(k), wm = weight_int(km);
-          u.y = to_fixed(xk[i].x, sc, wk);
-          w.y = to_fixed(xm[i].x, sc, wm);
+          u.y = to_fixed(xk[i].x, su, wk);
+          w.y = to_fixed(xm[i].x, su, wm);
           wk.neg = wm.neg = true;
-          u.x = to_fixed(xk[i].y, sc, wk);
-          w.x = to_fixed(xm[i].y, sc, wm);
+          u.x = to_fixed(xk[i].y, su, wk);
+          w.x = to_fixed(xm[i].y, su, wm);
         } else {
           const Weight one = weight_one();
-          u = Fx{to_fixed(xk[i].x, sc, one), to_fixed(xk[i].y, sc, one)};
-          w = Fx{to_fixed(xm[i].x, sc, one), to_fixed(xm[i].y, sc, one)};
+          u = Fx{to_fixed(xk[i].x, su, one), to_fixed(xk[i].y, su, one)};
+          w = Fx{to_fixed(xm[i].x, su, one), to_fixed(xm[i].y, su, one)};
         }
         if (k == 0) {  // X_{N/2} = 0; the self-paired X_{M/2}: Z = 2 conj X
           // S = X_0, D = X_0, Z = X_0 + i X_0
-          st(0, Fx{u.x - u.y, u.x + u.y});
-          st(M / 2, Fx{2 * w.x, -2 * w.y});
+          put(0, Fx{u.x - u.y, u.x + u.y});
+          put(M / 2, Fx{2 * w.x, -2 * w.y});
         } else {
           const Fx s = {u.x + w.x, u.y - w.y}, d = {u.x - w.x, u.y + w.y};
           const Fx q = mul_pi(cmulc(d, __ldg(twf + k)));  // Z_k = S + i D conj w
-          st(k, Fx{s.x + q.x, s.y + q.y});
-          st(M - k, Fx{s.x - q.x, q.y - s.y});  // conj(S - i D conj w)
+          put(k, Fx{s.x + q.x, s.y + q.y});
+          put(M - k, Fx{s.x - q.x, q.y - s.y});  // conj(S - i D conj w)
         }
       }
     }
