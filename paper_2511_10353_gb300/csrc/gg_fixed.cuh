@@ -39,6 +39,14 @@ __device__ __forceinline__ long long mul_real(long long a, int h, int l) {
   const int al = lo_of(a), ah = hi_of(a);
   return join((long long)ah * h, wide(al, h, wide(ah, l, kRound)));
 }
+// a / 2, halves to even. Cut off, a quarter of a unit would be lost on average, the
+// same everywhere; the transforms along the other axes gather such a constant in
+// single modes and cells (1536^3, forward and back: one cell off by 2000 times the
+// rms error).
+__device__ __forceinline__ long long half_even(long long a) {
+  const long long h = a >> 1;
+  return h + (long long)((uint32_t)a & (uint32_t)h & 1u);
+}
 // An integer, times 2^-s, rounded to FP64 without the FP64 pipe: normalised,
 // rounded to nearest even and put together by integers (26 instructions; two exact
 // halves and two FP64 additions, 32 cycles of that pipe, took 13.9 instead of

@@ -14,8 +14,9 @@
 // the sum of |re| + |im|, above N = 768 more closely (modulus): the largest one for
 // which that stays below 2^62.5. Every intermediate and output of the transform is
 // bounded by A (all twiddles have modulus one), and the sums re + im that products
-// by (1 + i) / sqrt(2) take by sqrt(2) A, so nothing reaches 2^63. (z forward, whose
-// last step adds two outputs, and the i m outputs of the strided passes: 2^62.)
+// by (1 + i) / sqrt(2) take by sqrt(2) A, so nothing reaches 2^63. (The i m outputs of the
+// strided passes 2^62; z forward, whose last step adds two outputs, 2^61, above N =
+// 512, where that bit counts, 2^62 and the outputs halved first.)
 //
 // Rounding the inputs to their unit u changes each output by 0.41 sqrt(N) u rms.
 // The unit is A 2^-62.5 to A 2^-61.5 and A <= sqrt(N) L2 (L2: root of the sum of
@@ -29,6 +30,8 @@
 //   N             64    256   384   512   768   1024  1536
 //   fixed point   1.5   1.6   2.8   2.2   3.4   3.0   4.4   e-16 relative L2 (largest: 4.7)
 //   FP64          4.3   5.4   5.8   5.7   6.2   6.2   6.6
+// Every rounding is unbiased: the modes along the axes are off by 1.5e-16 to 4.6e-16
+// (FP64: 2.7e-16 to 5.6e-16), the worst cell by 6 to 11 times the rms error.
 // Measured against 113-bit arithmetic, the density chain of six transforms is
 // off by 1.2e-16 to 2.7e-16 relative L2 (white, steep, spike and single-mode
 // fields of 32^3 to 128^3; the FP64 transforms: 3.0e-16 to 5.2e-16).
@@ -58,7 +61,7 @@ template <bool INV> struct Butterfly<3, INV, Fx> {
   static __device__ __forceinline__ void run(Fx *v) {
     constexpr int h = fx::high_half(fx::kSin60), l = fx::low_half(fx::kSin60);
     const Fx s = cadd(v[1], v[2]), d = csub(v[1], v[2]);
-    const Fx t = {v[0].x - (s.x >> 1), v[0].y - (s.y >> 1)};
+    const Fx t = {v[0].x - fx::half_even(s.x), v[0].y - fx::half_even(s.y)};
     const Fx r = mul_wi<INV>(Fx{fx::mul_real(d.x, h, l), fx::mul_real(d.y, h, l)});
     v[0] = cadd(v[0], s);
     v[1] = cadd(t, r);

@@ -368,6 +368,7 @@ __global__ void __launch_bounds__(ZShape<N>::THREADS,
   using Sh = ZShape<N>;
   constexpr int M = Sh::M, K = Sh::K, E = Sh::E, P = Sh::P, L = Sh::L, S = ct::nstages(K);
   constexpr int RF = ct::radix_of(K, 0, false), SPANF = M / RF, NBF = E / RF;
+  constexpr bool HALVE = N > 512;  // see the head of gg_fx.cuh
   extern __shared__ __align__(128) unsigned char smem_raw[];
   uint64_t *bar = reinterpret_cast<uint64_t *>(smem_raw);
   int2 *parts = reinterpret_cast<int2 *>(smem_raw + 128);
@@ -441,7 +442,7 @@ __global__ void __launch_bounds__(ZShape<N>::THREADS,
             float s = 0.0f;
 #pragma unroll
             for (int i = 0; i < E; ++i) s += modulus<N>(d[i], e);
-            return s;  // the pairs' sums Z_k + conj Z_{M-k} are twice as large
+            return HALVE ? s : 2.0f * s;
           });  // its barrier: every thread has read its values
       if constexpr (NOISE) {
         if (tid == 0 && t + gridDim.x < ntiles) {
@@ -461,9 +462,12 @@ __global__ void __launch_bounds__(ZShape<N>::THREADS,
     }
     __syncthreads();
     ct::stages<I, M, E, false, 1, S>(p, tw, ld, st);
-    // the real-input spectrum by conjugate pairs, halves taken first so that
-    // every sum stays below 2^63: X_k = S/2 - i (D/2) w_k, X_{M-k} = conj(S/2 + i (D/2) w_k)
+    // the real-input spectrum by conjugate pairs: X_k = S/2 - i (D/2) w_k, X_{M-k} =
+    // conj(S/2 + i (D/2) w_k), S and D twice their bound
     double2 *dst = reinterpret_cast<double2 *>(a.out) + line * M;
+    auto part = [](I q) { return HALVE ? half_even(q) : q; };
+    Scale so = sc;
+    if constexpr (!HALVE) ++so.s;
 #pragma unroll
     for (int i = 0; i < E / 2; ++i) {
       const int k = p + P * i;
@@ -474,10 +478,10 @@ __global__ void __launch_bounds__(ZShape<N>::THREADS,
         dst[M / 2] = to_double2(Fx{zh.x, -zh.y}, sc);
       } else {
         const Fx zm = ld(M - k);
-        const Fx s = {(zk.x + zm.x) >> 1, (zk.y - zm.y) >> 1};
-        const Fx d = cmul(Fx{(zk.x - zm.x) >> 1, (zk.y + zm.y) >> 1}, __ldg(twf + k));
-        dst[k] = to_double2(Fx{s.x + d.y, s.y - d.x}, sc);
-        dst[M - k] = to_double2(Fx{s.x - d.y, -(s.y + d.x)}, sc);
+        const Fx s = {part(zk.x + zm.x), part(zk.y - zm.y)};
+        const Fx d = cmul(Fx{part(zk.x - zm.x), part(zk.y + zm.y)}, __ldg(twf + k));
+        dst[k] = to_double2(Fx{s.x + d.y, s.y - d.x}, so);
+        dst[M - k] = to_double2(Fx{s.x - d.y, -(s.y + d.x)}, so);
       }
     }
     __syncthreads();  // the work tile is rewritten next tile
@@ -488,8 +492,8 @@ __global__ void __launch_bounds__(ZShape<N>::THREADS,
 // pre-processing, Z_k = S + T and Z_{M-k} = conj(S - T), has |Z_k|^2 + |Z_{M-k}|^2 =
 // 4 (|X_k|^2 + |X_{M-k}|^2): the line's sum of moduli grows by at most 2 sqrt(2),
 // and each value fits far below it. Lines above 384 (N > 768) form the pairs in a
-// finer unit (2^-g of the transform's, g from the line: six bits on a flat spectrum)
-// and round them once, so that the transform's inputs carry one rounding at its
+// finer unit (2^-6 of the transform's where the line leaves room, as a flat spectrum
+// does) and round them once, so that the transform's inputs carry one rounding at its
 // unit instead of those of four inputs, which alone came to 5e-16 at N = 1536. At N =
 // 512 (2.9e-16 for six transforms without it) it would cost 1.5% of the run.
 __host__ __device__ constexpr int im_bits(int m) {  // frequencies below m are below 2^im_bits
@@ -577,11 +581,12 @@ __global__ void __launch_bounds__(ZShape<N>::THREADS, ZShape<N>::ctas(ZShape<N>:
       int g = 0;
       if constexpr (fine(N)) {  // weighted inputs stay below 2^60 in the finer unit
         const int room = 1082 - sc.s - sc.e - (im ? im_bits(M) : 0);
-        g = room < 0 ? 0 : (room < 6 ? room : 6);
+        g = room < 6 ? 0 : 6;
         su.k -= g;
       }
-      const I half = (1ll << g) >> 1;
-      auto put = [&](int n, Fx v) { st(n, Fx{(v.x + half) >> g, (v.y + half) >> g}); };
+      const I low = ((1ll << g) - 1) >> 1, tie = g ? 1 : 0;
+      auto round = [&](I q) { return (q + low + ((q >> g) & tie)) >> g; };  // halves to even
+      auto put = [&](int n, Fx v) { st(n, Fx{round(v.x), round(v.y)}); };
 #pragma unroll
       for (int i = 0; i < E / 2; ++i) {
         const int k = p + P * i, km = k ? M - k : M / 2;

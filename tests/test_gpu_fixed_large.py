@@ -58,6 +58,39 @@ def test_forward_and_back(gg, n):
     torch.cuda.empty_cache()
 
 
+@pytest.mark.parametrize("n", [96, 192, 384, 512, 768, 1024, 1536])
+def test_no_systematic_rounding(gg, n):
+    """Errors of one sign add up in single modes and cells: the modes along the axes
+    keep the bound of the whole field, and no cell is off by more than 12 times the
+    rms error (normal errors: 6.3 times among 1536^3)."""
+    plan = gg.Plan(n, float(n), BBKS, 50.0, "f64")
+    f = _white(n)
+    out = plan.smooth(f, 0.0)
+    plan.sync()
+    plan.close()
+    sign = 1.0 - 2.0 * (torch.arange(n, device="cuda", dtype=torch.float64) % 2)
+    mx = sum(f[i] * float(sign[i]) for i in range(n)) / n
+    err = [torch.zeros(n, dtype=torch.float64, device="cuda") for _ in range(3)]
+    ref = [torch.zeros(n, dtype=torch.float64, device="cuda") for _ in range(3)]
+    num = worst = 0.0
+    for i in range(n):
+        w = f[i] - float(sign[i]) * mx
+        w = w - sign[:, None] * (sign[:, None] * w).mean(0)[None, :]
+        w = w - sign[None, :] * (sign[None, :] * w).mean(1)[:, None]
+        d = out[i] - w
+        num += float((d ** 2).sum())
+        worst = max(worst, float(d.abs().max()))
+        for s, v in ((err, d), (ref, w)):
+            s[0][i] = v.sum()
+            s[1] += v.sum(1)
+            s[2] += v.sum(0)
+    assert worst < 12 * (num / n ** 3) ** 0.5
+    for e, r in zip(err, ref):
+        assert float((e - e.mean()).norm() / (r - r.mean()).norm()) < 6e-16
+    del f, out
+    torch.cuda.empty_cache()
+
+
 @pytest.mark.parametrize("n", [768, 1024])
 def test_displacement_against_fft(gg, n):
     """psi of caller noise against FP64 transforms of another library, 1e-12."""
