@@ -145,16 +145,16 @@ __device__ __forceinline__ Weight weight_int(int f) {  // |f| < 2^11
 }
 __device__ __forceinline__ long long to_fixed(double v, const Scale &sc, const Weight &w) {
   const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
-  const int e = (int)((hi >> 20) & 0x7ffu);
-  const uint32_t mh = (hi & 0xfffffu) | 0x100000u;
+  // a zero or subnormal has no leading bit and the exponent of a field of 1
+  const uint32_t field = (hi >> 20) & 0x7ffu, lead = min(field, 1u);
+  const uint32_t mh = (hi & 0xfffffu) + (lead << 20);
   const unsigned long long p = (unsigned long long)lo * w.m;
   const unsigned long long m = p + ((unsigned long long)(mh * w.m) << 32);
-  // m >= 2^62 and the result is below 2^62: r >= 0, except for a value dropped by
+  // m >= 2^62 (normal values) and the result is below 2^62: r >= 0, except for a value dropped by
   // its weight (m = 0), whose r may be anything. Rounded to nearest: cutting off
   // would shrink every transform by up to 2^-53.
-  const uint32_t r = min((uint32_t)(sc.k + w.c - e - 1), 63u);
-  unsigned long long f = ((m >> r) + 1) >> 1;
-  if (e == 0) f = 0;  // zeros and subnormals
+  const uint32_t r = min((uint32_t)(sc.k + w.c - 2) - field + lead, 63u);
+  const unsigned long long f = ((m >> r) + 1) >> 1;
   const long long g = (long long)f;
   return ((int)hi < 0) != w.neg ? -g : g;
 }

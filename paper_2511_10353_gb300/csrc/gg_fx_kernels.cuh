@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(AxisShape<N>::THREADS, AxisShape<N>::MINB)
           for (int r = 0; r < RF; ++r) d[b * RF + r] = bufd[(p + P * b + r * SPANF) * B + c];
         sc = scale(
             [&]() {
-              int e = 0;
+              int e = 1;
 #pragma unroll
               for (int i = 0; i < E; ++i) e = max_exp(e, d[i]);
               return e;
@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(AxisShape<N>::THREADS, AxisShape<N>::MINB)
       if (tid == 0) bulk_wait_read0();
       const Scale sc = scale(
           [&]() {
-            int e = 0;
+            int e = 1;
 #pragma unroll
             for (int i = 0; i < E; ++i) {
               const int x = max_exp(0, X[i]);
@@ -433,7 +433,7 @@ __global__ void __launch_bounds__(ZShape<N>::THREADS,
       sc = line_scale<N, true>(
           tid, l, p, parts,
           [&]() {
-            int e = 0;
+            int e = 1;
 #pragma unroll
             for (int i = 0; i < E; ++i) e = max_exp(e, d[i]);
             return e;
@@ -554,7 +554,7 @@ __global__ void __launch_bounds__(ZShape<N>::THREADS, ZShape<N>::ctas(ZShape<N>:
       sc = line_scale<N, true>(
           tid, l, p, parts,
           [&]() {
-            int e = 0;
+            int e = 1;
 #pragma unroll
             for (int i = 0; i < E / 2; ++i) {
               const int x = max_exp(0, xk[i]);
