@@ -220,8 +220,9 @@ gg_status gg_plan_set_variants(gg_plan_t *plan, const int32_t v[6]);
  * 1 chunk-major [k_z chunk][x][y][tile width], in which a tile of the x pass spans a few hundred kilobytes
  * per chunk instead of one memory page per row. Results are bit-identical
  * (same arithmetic in the same order). The chunk-major layout needs the four
- * strided passes' variants to share a tile width; otherwise the plain one
- * runs. gg_autotune chooses between them; gg_plan_layout reports the layout
+ * strided passes' variants to share a tile width. A plan whose variants were
+ * neither set nor tuned takes variants that do with layout 1 (its default ones
+ * again with layout 0); otherwise the plain layout runs. gg_autotune chooses between them; gg_plan_layout reports the layout
  * the next run takes (1 only where the chunk-major one applies). */
 gg_status gg_plan_set_layout(gg_plan_t *plan, int32_t chunked);
 gg_status gg_plan_layout(const gg_plan_t *plan, int32_t *out);

@@ -73,6 +73,8 @@ struct gg_plan {
   // the passes of a call overlap their launches (default_shapes); the batched
   // form's do not: its groups run on several streams and are captured
   int overlap = 0;
+  // the variants are default_shapes' (gg_plan_set_variants and gg_autotune choose others)
+  bool default_variants = true;
   int chunked = 0;  // 1: the three-component chain keeps the spectrum chunk-major (gg_plan_set_layout)
   // fault test (gg_test_arm_fault): the next y forward pass issues no copies
   int test_skip_copy = 0;
@@ -433,16 +435,20 @@ void choose_tiles(gg_plan_t *plan) {
 //   the integer pipes of the others idle (a run, FP64: 32: 84 -> 75; 64: 90.5 ->
 //   85.5; 96: 165 -> 188; 192: 811 -> 857; FP32: 32: 43 -> 33; 64: 43 -> 33; 96:
 //   56 -> 52; 144: 101 -> 90; 216: 261 -> 243; 256: 292 -> 277).
+void default_variants(gg_plan_t *plan) {
+  const int n = (int)plan->p.n;
+  if (plan->real_bytes != 4 || !gg::spec_tuned<float>(n)) return;
+  plan->variant[0] = plan->variant[5] = n <= 256 ? 3 : 2;
+  plan->variant[2] = gg::spec_three_ctas<float>(n) ? 2 : 0;
+  plan->variant[3] = n > 256 && n < 512 ? 1 : 0;
+  plan->variant[4] = n > 256 && n <= 512 ? 1 : 0;
+}
 void default_shapes(gg_plan_t *plan) {
   const int n = (int)plan->p.n;
   plan->overlap = plan->real_bytes == 4 || n <= 64;
   if (plan->real_bytes != 4 || !gg::spec_has<float>(n)) return;
   plan->chunked = (int64_t)n * (n / 2) * 8 >= ((int64_t)2 << 20);
-  if (!gg::spec_tuned<float>(n)) return;
-  plan->variant[0] = plan->variant[5] = n <= 256 ? 3 : 2;
-  plan->variant[2] = gg::spec_three_ctas<float>(n) ? 2 : 0;
-  plan->variant[3] = n > 256 && n < 512 ? 1 : 0;
-  plan->variant[4] = n > 256 && n <= 512 ? 1 : 0;
+  default_variants(plan);
 }
 
 void release(gg_plan_t *plan) {
@@ -672,6 +678,11 @@ int chunk_cols(gg_plan_t *plan) {
   for (int i = 2; i <= 4; ++i)
     if (gg::spec_axis_cols<R>(n, plan->variant[i]) != b) return 0;
   return b;
+}
+
+int layout_cols(const gg_plan_t *plan) {
+  gg_plan_t *p = const_cast<gg_plan_t *>(plan);
+  return plan->real_bytes == 8 ? chunk_cols<double>(p) : chunk_cols<float>(p);
 }
 
 // All three components with the spectrum chunk-major between the y forward
@@ -1030,6 +1041,7 @@ gg_status autotune(gg_plan_t *plan, int reps) {
     plan->prof_launches[k] = 0;
   }
   for (int i = 0; i < 6; ++i) plan->variant[i] = best_v[i];
+  plan->default_variants = false;
   // the layout between the y passes: chunk-major where the chosen strided
   // variants share a tile width and the whole three-component step is faster
   plan->chunked = 0;
@@ -2094,19 +2106,26 @@ gg_status gg_plan_set_variants(gg_plan_t *plan, const int32_t v[6]) {
     if (v[i] < 0 || v[i] >= nv) return fail(plan, GG_EINVAL, "variant out of range");
   }
   for (int i = 0; i < 6; ++i) plan->variant[i] = v[i];
+  plan->default_variants = false;
   return GG_OK;
 }
 
 gg_status gg_plan_set_layout(gg_plan_t *plan, int32_t chunked) {
   if (!plan || (chunked != 0 && chunked != 1)) return fail(plan, GG_EINVAL, "plan NULL or layout not 0/1");
   plan->chunked = chunked;
+  // At 384 and 512 the default strided variants differ in tile width, which the
+  // chunk-major layout cannot have: variant 0 of each shares one.
+  if (plan->default_variants) {
+    default_variants(plan);
+    if (chunked && layout_cols(plan) == 0)
+      for (int i = 1; i < 5; ++i) plan->variant[i] = 0;
+  }
   return GG_OK;
 }
 
 gg_status gg_plan_layout(const gg_plan_t *plan, int32_t *out) {
   if (!plan || !out) return fail(nullptr, GG_EINVAL, "plan or out is NULL");
-  *out = plan->chunked && (plan->real_bytes == 8 ? chunk_cols<double>(const_cast<gg_plan_t *>(plan))
-                                                 : chunk_cols<float>(const_cast<gg_plan_t *>(plan))) > 0;
+  *out = plan->chunked && layout_cols(plan) > 0;
   return GG_OK;
 }
 
