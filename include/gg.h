@@ -199,8 +199,9 @@ gg_status gg_profile_read(gg_plan_t *plan, int reset, int *count, const char **n
  * Runs the whole path `reps` times per tile variant on the plan's own buffers
  * (allocating the component workspaces and one scratch grid for the call),
  * times each pass with CUDA events and keeps the fastest variant per pass for
- * later calls. Synchronous. Other sizes, and FP64, have one shape: returns
- * GG_OK and changes nothing.
+ * later calls, then the faster layout (gg_plan_set_layout). FP64 sizes with
+ * specialised kernels have one shape, and the layout alone is timed.
+ * Synchronous. Other sizes: returns GG_OK and changes nothing.
  * Results do not depend on the variant (same arithmetic, different tiling). */
 gg_status gg_autotune(gg_plan_t *plan, int reps);
 

@@ -987,8 +987,11 @@ gg_status run_host(gg_plan_t *plan, uint64_t seed, const void *noise_host, void 
 // kind map below picks each pass's time.
 template <typename R>
 gg_status autotune(gg_plan_t *plan, int reps) {
-  if (!gg::spec_tuned<R>((int)plan->p.n)) return GG_OK;
-  gg_status st;
+  const int n = (int)plan->p.n;
+  // FP64 has one tile shape a size: its layout alone is chosen
+  const bool shapes = gg::spec_tuned<R>(n);
+  if (!shapes && !(sizeof(R) == 8 && gg::spec_has<R>(n))) return GG_OK;
+  gg_status st = GG_OK;
   if ((st = ensure_grid(plan, &plan->work2)) != GG_OK) return st;
   if ((st = ensure_grid(plan, &plan->work3)) != GG_OK) return st;
   void *tmp = nullptr;
@@ -1011,7 +1014,7 @@ gg_status autotune(gg_plan_t *plan, int reps) {
   // 1536^3 variant 3 chosen, in which pos + vel takes 22.9 ms against 21.8 in 2)
   void *pos[3] = {tmp, tmp, tmp}, *vel[3] = {tmp, tmp, tmp};
   const int vmax = std::max(gg::kSpecZVariants, gg::kSpecAxisVariants);
-  for (int v = 0; v < vmax; ++v) {
+  for (int v = 0; shapes && v < vmax; ++v) {
     for (int i = 0; i < 6; ++i) plan->variant[i] = v < nvar[i] ? v : 0;
     plan->prof_on = false;
     if ((st = run_zeldovich<R>(plan, 1, nullptr, nullptr, pos, vel)) != GG_OK) break;  // warm
@@ -1040,8 +1043,10 @@ gg_status autotune(gg_plan_t *plan, int reps) {
     plan->prof_ms[k] = 0;
     plan->prof_launches[k] = 0;
   }
-  for (int i = 0; i < 6; ++i) plan->variant[i] = best_v[i];
-  plan->default_variants = false;
+  if (shapes) {
+    for (int i = 0; i < 6; ++i) plan->variant[i] = best_v[i];
+    plan->default_variants = false;
+  }
   // the layout between the y passes: chunk-major where the chosen strided
   // variants share a tile width and the whole three-component step is faster
   plan->chunked = 0;
