@@ -1376,13 +1376,17 @@ gg_status run_moments(gg_plan_t *plan, const void *field, double out[4]) {
     return cuda_fail(plan, e, "field moments");
   const double *first = h.data() + 3 * (size_t)blocks;
   const double mean = first[0];
-  double dev = 0.0;
-  for (int b = 0; b < blocks; ++b) dev += first[3 + 3 * b];
-  double var = dev / (double)count;
-  if (sizeof(R) == 4) {  // deviations from the FP32 value nearest to the mean
-    const double off = mean - (double)(float)mean;
-    var -= off * off;
+  double dev = 0.0, rest = 0.0, lin = 0.0;
+  for (int b = 0; b < blocks; ++b) {
+    const double v = first[3 + 3 * b], t = dev + v, w = t - dev;
+    rest += (dev - (t - w)) + (v - w);  // what the addition lost, exactly
+    dev = t;
+    lin += first[4 + 3 * b];
   }
+  // FP32: deviations from the FP32 value nearest to the mean, less their own mean
+  if (std::isfinite(rest)) dev += rest;
+  if (sizeof(R) == 4) dev -= lin / (double)count * lin;
+  const double var = dev / (double)count;
   out[0] = mean;
   out[1] = var;
   out[2] = first[1];

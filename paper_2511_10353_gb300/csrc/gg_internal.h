@@ -235,7 +235,7 @@ struct MomentArgs {
   int64_t count;
   // device, 6 blocks + 3: first pass [blocks][sum, min, max], {mean, min, max},
   // second pass [blocks][sum of squared deviations from the mean (FP32 fields:
-  // from the FP32 value nearest to it), -, -]
+  // from the FP32 value nearest to it), sum of those deviations (FP32), -]
   double *slots;
 };
 // Both passes and the mean between them, on s.

@@ -17,11 +17,12 @@
 // bound by the FP64 rate (512^3 1537 us a pass, 20 times the read), so a
 // thread adds 32 values exactly, as 64-bit integers in units of 2^-55 of
 // their largest binary order, and makes one FP64 addition of them. The second
-// pass squares d = v - c for the FP32 value c nearest to the mean, with
-// d = hi + lo and hi^2 = p + e exact: the p add up as integers too, the
-// e + 2 hi lo (below 2^-23 p) in FP32, and sum (v - mean)^2 =
-// sum d^2 - count (mean - c)^2. Groups that hold an infinity, a NaN or only
-// tiny values add in FP64. 512^3: 132 and 163 us.
+// pass does the same with the squares of d = v - c for the FP32 value c nearest to
+// the mean: d is an integer in units of 2^-58 of the group's largest order, squared
+// by its halves (three multiply-adds), and
+// sum (v - mean)^2 = sum d^2 - (sum d)^2 / count. (Squares in FP32 with their
+// rounding errors added beside them were off by up to 3e-15.) Groups that hold an
+// infinity or a NaN add in FP64. 512^3: 132 and 186 us (squares in FP32 163).
 #include <cfloat>
 #include <cstdint>
 
@@ -136,6 +137,20 @@ __device__ __forceinline__ long long fixed32(float v, int E) {
   const long long f = (long long)(((unsigned long long)m << 32) >> (sh < 63 ? sh : 63));
   return (int)b < 0 ? -f : f;
 }
+// v in units of 2^(E - 184), modulo 2^64: v - c below 2^(E - 126) is then the exact
+// difference of two such values, below 2^58, however large v and c are themselves
+// (a value that the shift takes out of the word is a multiple of 2^64 units). Bits
+// below one unit (v below 2^-34 of that bound) are cut off.
+__device__ __forceinline__ long long units58(float v, int E) {
+  const uint32_t b = __float_as_uint(v);
+  const int field = (int)((b >> 23) & 255u), lead = min(field, 1);
+  const int m = (int)((b & 0x7fffffu) + ((uint32_t)lead << 23));
+  const int sh = field + 1 - lead - E + 34;
+  const long long w = ((int)b < 0 ? -m : m) >> min(max(-sh, 0), 31);
+  long long f;  // shl.b64 clamps its shift at 64
+  asm("shl.b64 %0, %1, %2;" : "=l"(f) : "l"(w), "r"(max(sh, 0)));
+  return f;
+}
 __device__ __forceinline__ double unfixed(long long f, int E) {  // E >= 1
   return (double)f * __hiloint2double((E - 182 + 1023) << 20, 0);
 }
@@ -146,9 +161,9 @@ __device__ __forceinline__ int exponent_of(uint32_t bits) {
 
 constexpr int kMomentVec = 8;  // float4 a thread and group
 
-// The sum (SECOND: of squared deviations) of 32 FP32 values.
+// The sum of 32 FP32 values; SECOND: of the squares of d = v - c, and in `lin` of d.
 template <bool SECOND>
-__device__ __forceinline__ double group_sum(const float4 *v, float c) {
+__device__ __forceinline__ double group_sum(const float4 *v, float c, double &lin) {
   float x[4 * kMomentVec];
 #pragma unroll
   for (int i = 0; i < kMomentVec; ++i) {
@@ -172,37 +187,45 @@ __device__ __forceinline__ double group_sum(const float4 *v, float c) {
     for (int i = 0; i < 4 * kMomentVec; ++i) s += (double)x[i];
     return s;
   } else {
-    float p[4 * kMomentVec], t = 0.0f;
 #pragma unroll
-    for (int i = 0; i < 4 * kMomentVec; ++i) {
-      const float hi = __fsub_rn(x[i], c);  // x - c = hi + lo exactly
-      const float bp = __fsub_rn(hi, x[i]);
-      const float lo = __fsub_rn(__fsub_rn(x[i], __fsub_rn(hi, bp)), __fadd_rn(c, bp));
-      p[i] = __fmul_rn(hi, hi);
-      t = __fadd_rn(t, fmaf(2.0f * hi, lo, fmaf(hi, hi, -p[i])));
-      top = max(top, __float_as_uint(p[i]));
-    }
-    // below 2^-67 the remainders e would underflow
-    if (top < 0x7f800000u && top >= (60u << 23)) {
-      const int E = exponent_of(top);
-      long long s = 0;
+    for (int i = 0; i < 4 * kMomentVec; ++i)
+      top = max(top, __float_as_uint(__fsub_rn(x[i], c)) & 0x7fffffffu);
+    if (top < 0x7f800000u) {
+      // of the largest |d|, below 1 for subnormals
+      const int E = top >= 0x800000u ? (int)(top >> 23) : 9 - __clz((int)top);
+      const long long fc = units58(c, E);
+      // d = dh 2^32 + dl: the sums of d, dh^2, dh dl and (dl / 8)^2, each below 2^63
+      long long l = 0, hh = 0, hl = 0, ll = 0;
 #pragma unroll
-      for (int i = 0; i < 4 * kMomentVec; ++i) s += fixed32(p[i], E);
-      return unfixed(s, E) + (double)t;
+      for (int i = 0; i < 4 * kMomentVec; ++i) {
+        const long long d = units58(x[i], E) - fc;
+        const int dl = (int)(uint32_t)d, dh = (int)(d >> 32) + (int)((uint32_t)dl >> 31);
+        l += d;
+        hh += (long long)dh * dh;
+        hl += (long long)dh * dl;
+        ll += (long long)(dl >> 3) * (dl >> 3);
+      }
+      lin += (double)l * __hiloint2double((E - 184 + 1023) << 20, 0);
+      const long long t = (hh << 5) + (hl >> 26) + (ll >> 53);  // in units of 2^59
+      return (double)t * __hiloint2double((2 * E - 309 + 1023) << 20, 0);
     }
     double s = 0.0;
     for (int i = 0; i < 4 * kMomentVec; ++i) {
       const double d = (double)x[i] - (double)c;
       s += d * d;
+      lin += d;
     }
     return s;
   }
 }
 
+// {sum of s, minimum of lo, maximum of hi} of the CTA; LIN: lo adds up as s does.
+template <bool LIN> __device__ __forceinline__ double join_lo(double a, double b) { return LIN ? a + b : fmin(a, b); }
+template <bool LIN = false>
 __device__ __forceinline__ void block_slots(double s, double lo, double hi, double *slots) {
   for (int o = 16; o > 0; o >>= 1) {
     s += __shfl_xor_sync(0xffffffffu, s, o);
-    lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    lo = join_lo<LIN>(lo, __shfl_xor_sync(0xffffffffu, lo, o));
     hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
   }
   __shared__ double ws[3][8];
@@ -214,10 +237,10 @@ __device__ __forceinline__ void block_slots(double s, double lo, double hi, doub
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    double ts = 0.0, tl = DBL_MAX, th = -DBL_MAX;
+    double ts = 0.0, tl = LIN ? 0.0 : DBL_MAX, th = -DBL_MAX;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
       ts += ws[0][w];
-      tl = fmin(tl, ws[1][w]);
+      tl = join_lo<LIN>(tl, ws[1][w]);
       th = fmax(th, ws[2][w]);
     }
     slots[3 * blockIdx.x] = ts;
@@ -228,7 +251,7 @@ __device__ __forceinline__ void block_slots(double s, double lo, double hi, doub
 
 template <typename R, bool SECOND>
 __global__ void __launch_bounds__(256) k_moments(const MomentArgs a) {
-  double s = 0.0, lo = DBL_MAX, hi = -DBL_MAX;
+  double s = 0.0, lo = SECOND ? 0.0 : DBL_MAX, hi = -DBL_MAX;  // SECOND: lo sums the deviations
   const double mean = SECOND ? a.slots[3 * gridDim.x] : 0.0;  // k_moments_mean's
   if constexpr (sizeof(R) == 4) {
     const float4 *f = reinterpret_cast<const float4 *>(a.field);
@@ -242,7 +265,7 @@ __global__ void __launch_bounds__(256) k_moments(const MomentArgs a) {
       float4 v[kMomentVec];
 #pragma unroll
       for (int i = 0; i < kMomentVec; ++i) v[i] = __ldg(f + g * GROUP + i * 256 + threadIdx.x);
-      s += group_sum<SECOND>(v, c);
+      s += group_sum<SECOND>(v, c, lo);
       if constexpr (!SECOND) {
 #pragma unroll
         for (int i = 0; i < kMomentVec; ++i) {
@@ -257,11 +280,14 @@ __global__ void __launch_bounds__(256) k_moments(const MomentArgs a) {
       const float v = fs[i];
       const double d = SECOND ? (double)v - (double)c : (double)v;
       s += SECOND ? d * d : d;
+      if constexpr (SECOND) lo += d;
       flo = fminf(flo, v);
       fhi = fmaxf(fhi, v);
     }
-    lo = fmin(lo, (double)flo);
-    hi = fmax(hi, (double)fhi);
+    if constexpr (!SECOND) {
+      lo = fmin(lo, (double)flo);
+      hi = fmax(hi, (double)fhi);
+    }
   } else {
     const R *f = reinterpret_cast<const R *>(a.field);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.count;
@@ -275,7 +301,7 @@ __global__ void __launch_bounds__(256) k_moments(const MomentArgs a) {
       }
     }
   }
-  block_slots(s, lo, hi, a.slots + (SECOND ? 3 * gridDim.x + 3 : 0));
+  block_slots<SECOND>(s, lo, hi, a.slots + (SECOND ? 3 * gridDim.x + 3 : 0));
 }
 
 // The first pass's slots added in a fixed order: {mean, min, max} after them.
