@@ -36,8 +36,7 @@ namespace ct {
 // whole butterfly (n = 256: 16 x 16; n = 512: 32 x 16): each radix is one
 // DFT in registers (constant twiddles inside it), so a transform makes one
 // shared-memory round trip and one twiddle stage instead of two or three of
-// each. Other lengths, and every FP64 codelet (whose bound is the FP64
-// pipe, not the stage count), use radix 8 first, then 4 or 2, then the 3s.
+// each. Other lengths use radix 8 first, then 4 or 2, then the 3s.
 // The fixed-point codelets of the FP64 sizes (kFx, R = long long) keep a thread
 // at 8 or 12 elements (four registers each) where the length allows it.
 constexpr int kBig = 1 << 20, kFx = 1 << 21, kLine = 1 << 22;
@@ -315,9 +314,9 @@ template <typename T> __device__ __forceinline__ Tw<T, false> tw_global(const vo
 
 // Twiddles of a stage with NS > 1: FP32 radices up to 8 load w^1 per
 // butterfly (before the stage's shared-memory reads, to overlap their
-// latency) and form the other powers by at most three products; FP64, and
-// the large FP32 radices, read every power w^(k r) from the table (an FP32
-// power chain over 15 or 31 steps would lose accuracy).
+// latency) and form the other powers by at most three products; the large FP32
+// radices (a power chain over 15 or 31 steps would lose accuracy) and the
+// fixed-point codelets read every power w^(k r) from the table.
 template <typename R, int RAD> __host__ __device__ constexpr bool powers_from_w1() {
   return sizeof(R) == 4 && (RAD == 2 || RAD == 3 || RAD == 4 || RAD == 8);
 }
@@ -591,6 +590,7 @@ __host__ __device__ constexpr bool ct_tuned(int n) {
 }
 
 template <typename R, int N, int V> struct AxisPolicy {
+  static_assert(sizeof(R) == 4, "FP32; FP64 is fixed-point (gg_fx_kernels.cuh)");
   static constexpr bool TUNED = ct_tuned(N);
   static constexpr int CB = 2 * (int)sizeof(R);
   static constexpr bool BIG = is_big(skey<R>(N));
@@ -688,6 +688,7 @@ using LineT = typename std::conditional<
 // the stages (where each line lies within one warp; warps then drift apart),
 // variant 3 the lines of variant 1 with warp barriers.
 template <typename R, int N, int V> struct ZPolicy {
+  static_assert(sizeof(R) == 4, "FP32; FP64 is fixed-point (gg_fx_kernels.cuh)");
   static constexpr int M = N / 2;
   using T = LineT<R, M>;  // the lines' stage arithmetic
   static constexpr int E = elems(skey<T>(M));
@@ -698,9 +699,8 @@ template <typename R, int N, int V> struct ZPolicy {
   static constexpr bool FUSE = fuse_pair<T, M, E>();
   // Padding of the work tile, per direction: one empty slot every PAD values
   // (0: none). Chosen by counting the shared-memory wavefronts of every
-  // stage's stores and loads for each size; FP32 (FP64 keeps 1 in 16).
+  // stage's stores and loads for each size.
   static constexpr int pad_of(bool inv) {
-    if (sizeof(R) != 4) return 16;
     if (inv && FUSE) {             // register pair first: its stores are 12-24 apart
       if (M == 768) return 32;         // 248 wavefronts a line instead of 360 unpadded
       if (M == 192 || M == 96) return 64;
@@ -729,13 +729,12 @@ template <typename R, int N, int V> struct ZPolicy {
   static constexpr int WORK_FWD = L * LD_FWD;
   // CTAs per SM the register allocation must leave room for: enough for 16
   // warps, as far as the shared memory of the pass allows (inverse: a dense
-  // staging tile and the padded tile; forward: the padded tile). FP64 lines
-  // need twice the registers and run at the FP64 rate: no bound there.
+  // staging tile and the padded tile; forward: the padded tile)
   static constexpr int min_blocks(int smem) {
     if (V == kPersistV) return 2;
     const int by_smem = (228 * 1024) / smem, by_warps = 512 / THREADS;
     const int m = by_smem < by_warps ? by_smem : by_warps;
-    return sizeof(R) == 4 && m > 0 ? m : 1;
+    return m > 0 ? m : 1;
   }
   static constexpr int MINB_INV = min_blocks(128 + DENSE * CB + WORK_INV * CB);
   static constexpr int MINB_FWD = min_blocks(WORK_FWD * CB);
