@@ -339,9 +339,13 @@ gg_status gg_gaussian_field_static(const gg_params *p, uint64_t seed, const void
 /* Transpose of the linear map W -> psi_j (Eqs. 1-2) applied to upstream
  * gradients: g_noise = sum_j J_j^T g_psi[j]. Each J_j multiplies the spectrum
  * by the purely imaginary, Hermitian i k_j D sqrt(P/V) / k^2, so J_j^T = -J_j:
- * g_noise = -sum_j J_j g_psi[j], one forward chain per non-NULL component;
- * no transform intermediates are stored. g_psi entries: N^3 reals or NULL;
- * g_noise_dev: N^3 reals (overwritten). */
+ * g_noise = -sum_j J_j g_psi[j]. Three FP32 gradients at a size with specialised
+ * kernels are joined in the spectrum and take one inverse chain; otherwise one
+ * forward chain runs per non-NULL component. No transform intermediates are
+ * stored. g_psi entries: N^3 reals or NULL; g_noise_dev: N^3 reals, overwritten
+ * and used as scratch: it must not alias an entry of g_psi. The first call
+ * allocates component workspaces (one grid for the joined form, else as
+ * gg_zeldovich for the components given). */
 gg_status gg_zeldovich_adjoint(gg_plan_t *plan, const void *const g_psi_dev[3], void *g_noise_dev);
 
 /* Gaussian smoothing out = F^-1[exp(-k^2 R^2 / 2) F in] (R in Mpc/h, modes with

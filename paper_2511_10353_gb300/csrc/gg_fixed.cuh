@@ -25,7 +25,8 @@ __device__ __forceinline__ long long wide(int a, int b, long long c) { return (l
 __device__ __forceinline__ long long join(long long h, long long c) { return (h << 2) + (c >> 30); }
 constexpr long long kRound = 1ll << 29;
 
-// The low x low products (below half a unit) are left out.
+// The low x low products are left out: each a unit at most, a third of one rms and
+// without a bias.
 __device__ __forceinline__ Fx mul(Fx a, int rh, int rl, int ih, int il) {
   const int xl = lo_of(a.x), xh = hi_of(a.x), yl = lo_of(a.y), yh = hi_of(a.y);
   Fx o;

@@ -5,9 +5,9 @@
 // instructions a point, 14 SM cycles, however it is scheduled, and the FP64
 // kernels ran at 84% of that bound. The same transform on 64-bit integers takes
 // about 120 integer instructions a point, two to three cycles. 512^3 noise ->
-// pos + vel 59.1 -> 12.8 ms (z forward 12.9 -> 2.39, y 3.38 -> 0.90, x 11.1 -> 3.09,
-// y inverses 11.0 -> 2.67, z inverses 20.7 -> 3.68), bound by the latency of the
-// integer chains at 16 to 20 warps an SM.
+// pos + vel 59.1 -> 12.8 ms (z forward 12.9 -> 2.50, y 3.38 -> 0.90, x 11.1 -> 3.04,
+// y inverses 11.0 -> 2.63, z inverses 20.7 -> 3.74), bound by the latency of the
+// integer chains at 16 warps an SM (12 at 192 to 384, 8 at 768 and 1536).
 //
 // Each transform of N points (a column of a tile, a line) gets one power of two
 // as its scale, from the sum A of the moduli of its inputs, estimated from above by

@@ -2,7 +2,7 @@
 // arguments are 32-bit integers, so the logarithm, the sine and the cosine are
 // computed in 64-bit integers, and FP64 does the square root and the products
 // (8 instructions a pair instead of the 110 of log, sqrt and sincospi: the
-// 512^3 z forward pass 12.9 -> 2.39 ms together with its fixed-point transform).
+// 512^3 z forward pass 12.9 -> 2.50 ms together with its fixed-point transform).
 //
 // * ln u, u = (r + 1) 2^-32 = y 2^(-1-z), y in [1, 2) from the 32 bits: the top
 //   seven fraction bits select c ~ 1/y (11 bits), t = y c - 1 is exact, ln u =
